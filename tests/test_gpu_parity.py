@@ -643,6 +643,20 @@ def test_mg_vcycle_conductivity_map_matches_oracle():
     assert np.max(np.abs(z - z_ref)) <= 2e-5 * np.max(np.abs(z_ref))
 
 
+@pytest.mark.parametrize("nx,ny,L", [(1, 1, 1), (1, 8, 4), (8, 1, 10), (3, 7, 8), (8, 5, 10), (8, 8, 32)])
+def test_mg_coarsest_inverse(nx, ny, L):
+    """A single-level grid: the V-cycle is the coarsest level's exact solve, so the banded
+    device inverse (both orders of the in-plane sides, the widest band) is compared with a
+    dense solve.  FP32 coefficients, inverse entries and products: 64 products a lane."""
+    layers = [ti.si() if i % 2 == 0 else ti.bond() for i in range(L)]
+    st = ti.Stack(tuple(layers), h=1e4)
+    A = disc.assemble(nx, ny, st).toarray()
+    r = ti.random_vector(nx * ny * L, 23).astype(np.float32)
+    z = grid_of(nx, ny, st).precond(cuda(r), 0.0, precond="mg").cpu().double().numpy()
+    inv = np.linalg.inv(A)
+    assert np.all(np.abs(z - inv @ r) <= 1e-5 * (np.abs(inv) @ np.abs(r)))
+
+
 @pytest.mark.parametrize("graph", [0, 1])
 def test_mg_steady_solve(graph):
     st = ti.stack_c2()
