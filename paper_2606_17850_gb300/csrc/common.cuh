@@ -102,6 +102,16 @@ struct Ctl {
   double ad_rtrue_prev; // ||b - A x|| at the previous criterion evaluation (0: none)
 };
 
+// Start of every kernel of the solve chains (host side: th_launch).  They are launched
+// with programmatic serialisation: a kernel's blocks may become resident while the one
+// before it finishes, so the launch itself is off the critical path; the wait returns
+// once that kernel has completed and its writes are visible, so every kernel of a chain
+// waits before it touches memory.
+__device__ __forceinline__ void grid_dep_enter() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 template <typename T> __device__ __forceinline__ T ctl_alpha(const Ctl* c);
 template <> __device__ __forceinline__ float ctl_alpha<float>(const Ctl* c) { return __ldcg(&c->alpha_f); }
 template <> __device__ __forceinline__ double ctl_alpha<double>(const Ctl* c) { return __ldcg(&c->alpha_d); }

@@ -37,6 +37,7 @@ __global__ void k_ctl_reset(Ctl* c, CtlInit in) {
 // Start of a backward-Euler step: theta_n <- theta (element-wise) is done by
 // k_copy; this resets the per-step loop flags (counters keep accumulating).
 __global__ void k_step_begin(Ctl* c) {
+  grid_dep_enter();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   c->outer_done = 0;
   c->outer_it_step = 0;
@@ -46,6 +47,7 @@ __global__ void k_step_begin(Ctl* c) {
 }
 
 __global__ void k_step_end(Ctl* c) {
+  grid_dep_enter();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   c->step += 1;
   c->steps_done += 1;
@@ -55,6 +57,7 @@ __global__ void k_step_end(Ctl* c) {
 // which: 0 inner loop (!done), 1 outer loop (!outer_done), 2 step loop (step < n_steps,
 // and no fatal status).
 __global__ void k_cond(cudaGraphConditionalHandle h, const Ctl* c, int which) {
+  grid_dep_enter();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   unsigned v = 0;
   // TH_ECUDA (a bounded device wait ran out), TH_EBREAKDOWN, TH_ENONFINITE
@@ -85,6 +88,7 @@ __global__ void k_finalize(long long n, const double* __restrict__ theta, double
 }
 
 __global__ void k_copy64(long long n, const double* __restrict__ a, double* __restrict__ b) {
+  grid_dep_enter();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   b[i] = a[i];
@@ -113,6 +117,7 @@ __global__ void k_residual(Dims d, Ctl* ctl, Faces64 f, const LayerTab* tab, con
                            const TP* __restrict__ P, const TP* const* ptab, const double* __restrict__ theta_n,
                            TR* __restrict__ r, int mode, int count_outer, double* partials, int stride,
                            unsigned* counter) {
+  grid_dep_enter();
   if (mode != 2 && ld_int(&ctl->outer_done)) return;
   const Cell c = cell_of(d);
   if (ptab) P = ptab[ld_int(&ctl->map_idx)];
@@ -162,6 +167,7 @@ __global__ void k_finalize_df(long long n, const float* __restrict__ th_hi, cons
 
 __global__ void k_copy_df(long long n, const float* __restrict__ ah, const float* __restrict__ al,
                           float* __restrict__ bh, float* __restrict__ bl) {
+  grid_dep_enter();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   bh[i] = ah[i];
@@ -173,6 +179,7 @@ __global__ void k_copy_df(long long n, const float* __restrict__ ah, const float
 // entry.  The history array then holds theta_n for the whole step, so it also serves
 // as the step's theta_n (the right-hand side's C/dt T_n term).
 __global__ void k_step_extrap_df(long long n, float* th_hi, float* th_lo, float* thm_hi, float* thm_lo) {
+  grid_dep_enter();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const df cur = df_make(th_hi[i], th_lo[i]);
@@ -185,6 +192,7 @@ __global__ void k_step_extrap_df(long long n, float* th_hi, float* th_lo, float*
 }
 
 __global__ void k_step_extrap64(long long n, double* th, double* thn, double* thm) {
+  grid_dep_enter();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double cur = th[i];
@@ -196,6 +204,7 @@ __global__ void k_step_extrap64(long long n, double* th, double* thn, double* th
 // theta += ||r|| d in double-float.
 __global__ void k_theta_axpy_df(long long n, const Ctl* ctl, float* __restrict__ th_hi, float* __restrict__ th_lo,
                                 const float* __restrict__ d) {
+  grid_dep_enter();
   if (ld_int(&ctl->outer_done)) return;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -214,6 +223,7 @@ __global__ void k_residual_df(Dims d, Ctl* ctl, Faces32 gh, Faces32 gl, const La
                               const TP* const* ptab, const float* __restrict__ thn_hi,
                               const float* __restrict__ thn_lo, float* __restrict__ r, int count_outer,
                               double* partials, int stride, unsigned* counter) {
+  grid_dep_enter();
   if (ld_int(&ctl->outer_done)) return;
   const Cell c = cell_of(d);
   const TP* P = ptab[ld_int(&ctl->map_idx)];
@@ -282,6 +292,7 @@ __global__ void k_spmv_dot(Dims d, Ctl* ctl, const TC* __restrict__ gx, const TC
                            const TC* __restrict__ gz, const LayerTab* tab, const TV* __restrict__ z,
                            const TV* __restrict__ p_old, TV* __restrict__ p_new, TV* __restrict__ mu,
                            double* partials, int stride, unsigned* counter) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   const Cell c = cell_of(d);
   const int first = ld_int(&ctl->first);
@@ -309,6 +320,7 @@ template <typename TV, bool INIT, int ZMODE>
 __global__ void k_update(Dims d, Ctl* ctl, TV* __restrict__ x, const TV* __restrict__ p, TV* __restrict__ r,
                          const TV* __restrict__ mu, const TV* __restrict__ invd, TV* __restrict__ z, TV zscale,
                          int scaled, int rz_here, int scale_r, double* partials, int stride, unsigned* counter) {
+  grid_dep_enter();
   if (!INIT && ld_int(&ctl->done)) return;
   if (INIT && ld_int(&ctl->outer_done)) return;
   const Cell c = cell_of(d);
@@ -352,6 +364,7 @@ __global__ void k_cheb(Dims d, Ctl* ctl, const TC* __restrict__ gx, const TC* __
                        const TC* __restrict__ gz, const LayerTab* tab, const TV* __restrict__ r,
                        const TV* __restrict__ zprev, const TV* __restrict__ zcur, TV* __restrict__ znext,
                        const TV* __restrict__ invd, TV c1, TV c2, double* partials, int stride, unsigned* counter) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   const Cell c = cell_of(d);
   TV v[1] = {(TV)0};
@@ -410,6 +423,7 @@ __global__ void k_cheb64x(Dims d, Ctl* ctl, Faces64 f, const double* __restrict_
                           const double* __restrict__ zprev, const double* __restrict__ zcur,
                           double* __restrict__ znext, const double* __restrict__ invd, double c1, double c2,
                           double* partials, int stride, unsigned* counter) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   const Cell c = cell_of(d);
   double v[1] = {0.0};
@@ -437,6 +451,7 @@ __global__ void k_spmv_dot64x(Dims d, Ctl* ctl, Faces64 f, const double* __restr
                               const double* __restrict__ z, const double* __restrict__ p_old,
                               double* __restrict__ p_new, double* __restrict__ mu, double* partials, int stride,
                               unsigned* counter) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   const Cell c = cell_of(d);
   const int first = ld_int(&ctl->first);
@@ -462,6 +477,7 @@ template <typename TV>
 __global__ void k_zline(Dims d, Ctl* ctl, const float* __restrict__ gz, const float* __restrict__ zm,
                         const float* __restrict__ zc, const TV* __restrict__ r, TV* __restrict__ z,
                         double* partials, int stride, unsigned* counter) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   const int x = blockIdx.x * TH_BX + threadIdx.x;
   const int y = blockIdx.y * TH_BY + threadIdx.y;

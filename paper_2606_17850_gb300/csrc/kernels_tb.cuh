@@ -129,6 +129,7 @@ __global__ void __launch_bounds__(TB_EX * EY, 1)
               const __grid_constant__ CUtensorMap m_cur, const __grid_constant__ CUtensorMap m_prev,
               const __grid_constant__ CUtensorMap m_r, float* __restrict__ out_cur, float* __restrict__ out_prev,
               const __grid_constant__ TBParams<LMAX> P, double* partials, int stride, unsigned* counter) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   constexpr int H = STEPS;
   constexpr int TX = TB_EX - 2 * H, TY = EY - 2 * H;  // interior of a tile
@@ -347,6 +348,7 @@ __global__ void __launch_bounds__(TB_EX * TBF_EY, 1)
                const __grid_constant__ CUtensorMap m_gz, const float* __restrict__ invd, float* __restrict__ out_cur,
                float* __restrict__ out_prev, const __grid_constant__ TBFParams<LMAX> P, double* partials, int stride,
                unsigned* counter) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   constexpr int EY = TBF_EY;
   constexpr int H = STEPS;

@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(TH_BX* TH_BY4)
               const TC* __restrict__ gz, const LayerTab* tab, const float* __restrict__ r,
               const float* __restrict__ zprev, const float* __restrict__ zcur, float* __restrict__ znext, float c1,
               float c2, double* partials, int stride, unsigned* counter) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   const Walk4 w = walk4_of(d, zc);
   float part[1] = {0.f};
@@ -181,6 +182,7 @@ __global__ void __launch_bounds__(TH_BX* TH_BY4)
                   const float* __restrict__ gz, const LayerTab* tab, const float* __restrict__ z,
                   const float* __restrict__ p_old, float* __restrict__ p_new, float* __restrict__ mu,
                   double* partials, int stride, unsigned* counter) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   const int first = ld_int(&ctl->first);
   const float beta = first ? 0.f : ctl_beta<float>(ctl);
@@ -233,6 +235,7 @@ static __global__ void __launch_bounds__(256)
                 const float* __restrict__ mu, const float* __restrict__ invd, float* __restrict__ z, float zscale,
                 int scaled, int rz_here, int scale_r, double* partials, int stride, unsigned* counter, Dims d,
                 const LayerTab* tab) {
+  grid_dep_enter();
   if (!INIT && ld_int(&ctl->done)) return;
   if (INIT && ld_int(&ctl->outer_done)) return;
   const float alpha = INIT ? 0.f : ctl_alpha<float>(ctl);
@@ -338,6 +341,7 @@ __global__ void __launch_bounds__(TH_BX* TH_BY4, 2)
                      const float* __restrict__ th_hi, const float* __restrict__ th_lo, const TP* const* ptab,
                      const float* __restrict__ thn_hi, const float* __restrict__ thn_lo, float* __restrict__ r,
                      int count_outer, ResidInit ri, double* partials, int stride, unsigned* counter) {
+  grid_dep_enter();
   if (ld_int(&ctl->outer_done)) return;
   const TP* P = ptab[ld_int(&ctl->map_idx)];
   float v[3] = {0.f, 0.f, 0.f};
@@ -518,6 +522,7 @@ __global__ void __launch_bounds__(TH_BX* TH_BY4, 2)
 static __global__ void __launch_bounds__(256)
     k_theta_axpy_df_v4(long long n4, const Ctl* ctl, float* __restrict__ th_hi, float* __restrict__ th_lo,
                        const float* __restrict__ d) {
+  grid_dep_enter();
   if (ld_int(&ctl->outer_done)) return;
   const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= n4) return;
@@ -538,6 +543,7 @@ static __global__ void __launch_bounds__(256)
 // Start of a step with the extrapolated guess (see k_step_extrap_df).
 static __global__ void __launch_bounds__(256)
     k_step_extrap_df_v4(long long n4, float* th_hi, float* th_lo, float* thm_hi, float* thm_lo) {
+  grid_dep_enter();
   const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= n4) return;
   const long long i = 4 * q;
@@ -569,6 +575,7 @@ template <int ORD>
 static __global__ void __launch_bounds__(256)
     k_step_extrapq_df_v4(long long n4, const Ctl* ctl, float* th_hi, float* th_lo, float* thm_hi, float* thm_lo,
                          float* thm2_hi, float* thm2_lo, float* thm3_hi, float* thm3_lo) {
+  grid_dep_enter();
   const long long q4 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (q4 >= n4) return;
   const int step = ld_int(&ctl->step);

@@ -109,6 +109,7 @@ __global__ void __launch_bounds__(256) k_mg_smooth(const Ctl* ctl, MGDev v, cons
                                                    const float* __restrict__ b, const float* __restrict__ xin,
                                                    const float* __restrict__ xc, int nxc, int nyc,
                                                    float* __restrict__ xout, float omega) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -121,6 +122,7 @@ template <int LMAX, bool UNI>
 __global__ void __launch_bounds__(256) k_mg_restrict(const Ctl* ctl, MGDev v, const __grid_constant__ MGUni<LMAX> U,
                                                      const float* __restrict__ b, const float* __restrict__ x,
                                                      int nxc, int nyc, float* __restrict__ bc) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   __shared__ float rowsum[8][32];
   mg_restrict_tile<LMAX, UNI>(v, U, blockIdx.x, blockIdx.y, b, x, nxc, nyc, bc, rowsum);
@@ -167,6 +169,7 @@ __global__ void __launch_bounds__(256, 2) k_mg_smooth4(const Ctl* ctl, int nx, i
                                                        const float* __restrict__ b, const float* __restrict__ xin,
                                                        const float* __restrict__ xc, int nxc, int nyc,
                                                        float* __restrict__ xout, float omega) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -246,6 +249,7 @@ __global__ void __launch_bounds__(256) k_mg_restrict4(const Ctl* ctl, int nx, in
                                                       const __grid_constant__ MGUni<LMAX> U,
                                                       const float* __restrict__ b, const float* __restrict__ x,
                                                       int nxc, int nyc, float* __restrict__ bc) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   __shared__ float2 rowsum[LMAX][8][32];
   const int tx = threadIdx.x, ty = threadIdx.y;
@@ -344,6 +348,7 @@ __global__ void __launch_bounds__(32 * LMAX) k_mg_smooth_ct(const Ctl* ctl, int 
                                                            const float* __restrict__ xin,
                                                            const float* __restrict__ xc, int nxc, int nyc,
                                                            float* __restrict__ xout, float omega) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   __shared__ float sr[LMAX][32], sx[LMAX][32];
   const int t = threadIdx.x, z = threadIdx.y;
@@ -394,6 +399,7 @@ __global__ void __launch_bounds__(32 * LMAX) k_mg_restrict_ct(const Ctl* ctl, in
                                                              const float* __restrict__ b,
                                                              const float* __restrict__ x, int nxc, int nyc,
                                                              float* __restrict__ bc) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   __shared__ float sr[LMAX][32];
   const int t = threadIdx.x, z = threadIdx.y;
@@ -417,6 +423,7 @@ __global__ void __launch_bounds__(32 * LMAX) k_mg_restrict_ct(const Ctl* ctl, in
 // coarsest level: x = C b with the dense inverse C (n x n, FP32), a warp per row
 __global__ void __launch_bounds__(256) k_mg_coarsest(const Ctl* ctl, int n, const float* __restrict__ C,
                                                      const float* __restrict__ b, float* __restrict__ x) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   const int nw = blockDim.x >> 5;
   mg_coarsest_rows(n, C, b, x, blockIdx.x * nw + (threadIdx.x >> 5), nw * gridDim.x);
@@ -428,6 +435,7 @@ __global__ void __launch_bounds__(256) k_mg_coarsest(const Ctl* ctl, int n, cons
 __global__ void __launch_bounds__(256) k_mg_rz(long long n, Ctl* ctl, const float* __restrict__ r,
                                                const float* __restrict__ z, double* partials, int stride,
                                                unsigned* counter) {
+  grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   const long long step = (long long)gridDim.x * blockDim.x, t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long n4 = n / 4;
@@ -793,14 +801,13 @@ static th_status smooth(thermal_grid* g, int k, const float* b, const float* xin
   const MGLevelH& l = h->lv[k];
   const MGUni<LMAX> U = uni_of<LMAX>(h, k);
   if (mg_ct(g, k)) {
-    k_mg_smooth_ct<LMAX><<<dim3((l.nx + MG_CT_X - 1) / MG_CT_X, (l.ny + MG_CT_Y - 1) / MG_CT_Y), dim3(32, LMAX), 0,
-                           s>>>(g->ctl, l.nx, l.ny, g->L, U, b, xin, xc, nxc, nyc, xout, MG_OMEGA);
+    th_launch(k_mg_smooth_ct<LMAX>, dim3((l.nx + MG_CT_X - 1) / MG_CT_X, (l.ny + MG_CT_Y - 1) / MG_CT_Y), dim3(32, LMAX), 0, s, g->ctl, l.nx, l.ny, g->L, U, b, xin, xc, nxc, nyc, xout, MG_OMEGA);
     TH_CHECK_LAUNCH();
     return TH_OK;
   }
   if constexpr (LMAX == 8 || LMAX == 12) {
     if (mg_v4(g, k)) {
-      k_mg_smooth4<LMAX><<<dim3((l.nx / 4 + 31) / 32, (l.ny + 7) / 8), dim3(32, 8), 0, s>>>(g->ctl, l.nx, l.ny, g->L, U, b,
+      th_launch(k_mg_smooth4<LMAX>, dim3((l.nx / 4 + 31) / 32, (l.ny + 7) / 8), dim3(32, 8), 0, s, g->ctl, l.nx, l.ny, g->L, U, b,
                                                                                      xin, xc, nxc, nyc, xout,
                                                                                      MG_OMEGA);
       TH_CHECK_LAUNCH();
@@ -808,10 +815,10 @@ static th_status smooth(thermal_grid* g, int k, const float* b, const float* xin
     }
   }
   if (mg_uni(h, k))
-    k_mg_smooth<LMAX, true><<<col_grid(l.nx, l.ny), dim3(32, 8), 0, s>>>(g->ctl, dev_of(l, g->L), U, b, xin, xc, nxc,
+    th_launch(k_mg_smooth<LMAX, true>, col_grid(l.nx, l.ny), dim3(32, 8), 0, s, g->ctl, dev_of(l, g->L), U, b, xin, xc, nxc,
                                                                         nyc, xout, MG_OMEGA);
   else
-    k_mg_smooth<LMAX, false><<<col_grid(l.nx, l.ny), dim3(32, 8), 0, s>>>(g->ctl, dev_of(l, g->L), U, b, xin, xc,
+    th_launch(k_mg_smooth<LMAX, false>, col_grid(l.nx, l.ny), dim3(32, 8), 0, s, g->ctl, dev_of(l, g->L), U, b, xin, xc,
                                                                          nxc, nyc, xout, MG_OMEGA);
   TH_CHECK_LAUNCH();
   return TH_OK;
@@ -824,24 +831,23 @@ static th_status restrict_(thermal_grid* g, int k, const float* b, const float* 
   const MGLevelH& c = h->lv[k + 1];
   const MGUni<LMAX> U = uni_of<LMAX>(h, k);
   if (mg_ct(g, k)) {
-    k_mg_restrict_ct<LMAX><<<dim3((l.nx + MG_CT_X - 1) / MG_CT_X, (l.ny + MG_CT_Y - 1) / MG_CT_Y), dim3(32, LMAX), 0,
-                             s>>>(g->ctl, l.nx, l.ny, g->L, U, b, x, c.nx, c.ny, bc);
+    th_launch(k_mg_restrict_ct<LMAX>, dim3((l.nx + MG_CT_X - 1) / MG_CT_X, (l.ny + MG_CT_Y - 1) / MG_CT_Y), dim3(32, LMAX), 0, s, g->ctl, l.nx, l.ny, g->L, U, b, x, c.nx, c.ny, bc);
     TH_CHECK_LAUNCH();
     return TH_OK;
   }
   if constexpr (LMAX == 8 || LMAX == 12) {
     if (mg_v4(g, k)) {
-      k_mg_restrict4<LMAX><<<dim3((l.nx / 4 + 31) / 32, (l.ny + 7) / 8), dim3(32, 8), 0, s>>>(g->ctl, l.nx, l.ny, g->L, U,
+      th_launch(k_mg_restrict4<LMAX>, dim3((l.nx / 4 + 31) / 32, (l.ny + 7) / 8), dim3(32, 8), 0, s, g->ctl, l.nx, l.ny, g->L, U,
                                                                                        b, x, c.nx, c.ny, bc);
       TH_CHECK_LAUNCH();
       return TH_OK;
     }
   }
   if (mg_uni(h, k))
-    k_mg_restrict<LMAX, true><<<col_grid(l.nx, l.ny), dim3(32, 8), 0, s>>>(g->ctl, dev_of(l, g->L), U, b, x, c.nx,
+    th_launch(k_mg_restrict<LMAX, true>, col_grid(l.nx, l.ny), dim3(32, 8), 0, s, g->ctl, dev_of(l, g->L), U, b, x, c.nx,
                                                                           c.ny, bc);
   else
-    k_mg_restrict<LMAX, false><<<col_grid(l.nx, l.ny), dim3(32, 8), 0, s>>>(g->ctl, dev_of(l, g->L), U, b, x, c.nx,
+    th_launch(k_mg_restrict<LMAX, false>, col_grid(l.nx, l.ny), dim3(32, 8), 0, s, g->ctl, dev_of(l, g->L), U, b, x, c.nx,
                                                                            c.ny, bc);
   TH_CHECK_LAUNCH();
   return TH_OK;
@@ -869,7 +875,7 @@ th_status mg_vcycle(thermal_grid* g, const float* r, float* z, cudaStream_t s) {
   if (!h || !g->mg_valid) return th_fail(TH_ESTATE, "multigrid hierarchy not built");
   const int nl = (int)h->lv.size();
   if (nl == 1) {
-    k_mg_coarsest<<<(h->nc + 7) / 8, 256, 0, s>>>(g->ctl, h->nc, h->cinv, r, z);
+    th_launch(k_mg_coarsest, (h->nc + 7) / 8, 256, 0, s, g->ctl, h->nc, h->cinv, r, z);
     TH_CHECK_LAUNCH();
     return TH_OK;
   }
@@ -887,7 +893,7 @@ th_status mg_vcycle(thermal_grid* g, const float* r, float* z, cudaStream_t s) {
     TH_TRY(smooth_any(g, k, B[k], nullptr, nullptr, 1, 1, X[k], s));
     TH_TRY(restrict_any(g, k, B[k], X[k], h->lv[k + 1].b, s));
   }
-  k_mg_coarsest<<<(h->nc + 7) / 8, 256, 0, s>>>(g->ctl, h->nc, h->cinv, B[nl - 1], X[nl - 1]);
+  th_launch(k_mg_coarsest, (h->nc + 7) / 8, 256, 0, s, g->ctl, h->nc, h->cinv, B[nl - 1], X[nl - 1]);
   TH_CHECK_LAUNCH();
   for (int k = nl - 2; k >= 0; --k) {  // up: coarse correction (prolongated on the fly) + post-smooth
     const MGLevelH& c = h->lv[k + 1];
@@ -907,7 +913,7 @@ th_status mg_rz(thermal_grid* g, const float* r, const float* z, cudaStream_t s)
   const long long want = (n / 4 + 255) / 256;
   const int per = (dev >= 0 && dev < 64 && sms[dev] > 0) ? 4 * sms[dev] : 608;
   const unsigned nb = (unsigned)std::max(1LL, std::min<long long>(want, std::min(per, g->partials_stride)));
-  k_mg_rz<<<nb, 256, 0, s>>>(n, g->ctl, r, z, g->partials, g->partials_stride, g->counters);
+  th_launch(k_mg_rz, nb, 256, 0, s, n, g->ctl, r, z, g->partials, g->partials_stride, g->counters);
   TH_CHECK_LAUNCH();
   return TH_OK;
 }

@@ -254,7 +254,7 @@ static th_status tune_zchunk(thermal_grid* g, cudaStream_t s) {
     if (ci > 0 && zc == cands[ci - 1]) continue;
     const dim3 gb = v4_blocks(g, zc);
     auto run = [&]() {
-      TH_UNI(g->uniform, k_cheb_v4<float, true, false, U><<<gb, dim3(TH_BX, TH_BY4), 0, s>>>(
+      TH_UNI(g->uniform, th_launch(k_cheb_v4<float, true, false, U>, gb, dim3(TH_BX, TH_BY4), 0, s, 
                              d, zc, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz, g->tab, g->r32, g->zc32[0],
                              g->zc32[1], g->zc32[2], 0.5f, 0.5f, g->partials, g->partials_stride, g->counters));
     };
@@ -469,7 +469,7 @@ static th_status enq_update(const Plan& P, const VecSet<TV>& V, cudaStream_t st,
     if (P.v4) {
 #define TH_UPD4(ZM)                                                                                        \
   TH_UNI(P.uni && P.d.n < (1LL << 33),                                                                     \
-         k_update_v4<INIT, ZM, U><<<P.nbr4, 256, 0, st>>>(P.d.n / 4, ctl, xw, pp, V.r, V.mu, V.invd, V.zc[0], \
+         th_launch(k_update_v4<INIT, ZM, U>, P.nbr4, 256, 0, st, P.d.n / 4, ctl, xw, pp, V.r, V.mu, V.invd, V.zc[0], \
                                                           zs, P.scaled, rz1, scale_r, g->partials,          \
                                                           g->partials_stride, g->counters, P.d, g->tab))
       switch (P.pc) {
@@ -487,7 +487,7 @@ static th_status enq_update(const Plan& P, const VecSet<TV>& V, cudaStream_t st,
     }
   }
 #define TH_UPD(ZM)                                                                                          \
-  k_update<TV, INIT, ZM><<<P.gb, P.tb, 0, st>>>(P.d, ctl, xw, pp, V.r, V.mu, V.invd, V.zc[0], zs, P.scaled, \
+  th_launch(k_update<TV, INIT, ZM>, P.gb, P.tb, 0, st, P.d, ctl, xw, pp, V.r, V.mu, V.invd, V.zc[0], zs, P.scaled, \
                                                 rz1, scale_r, g->partials, g->partials_stride, g->counters)
   switch (P.pc) {
     case TH_PC_NONE: TH_UPD(0); break;
@@ -599,7 +599,7 @@ static th_status tb_launch(const Plan& P, const VecSet<float>& V, cudaStream_t s
                                (int)smem));
   const int nblk = std::min(ntiles, sm_count());
   if (nblk > g->partials_stride) return th_fail(TH_ESTATE, "partials buffer smaller than the temporal-blocking grid");
-  k_cheb_tb<LM, EY, ST, SC, LA, FI><<<nblk, dim3(TB_EX, EY), smem, st>>>(
+  th_launch(k_cheb_tb<LM, EY, ST, SC, LA, FI>, nblk, dim3(TB_EX, EY), smem, st, 
       P.d, ntx, ntiles, c.in_prev >= 0 ? 1 : 0, g->ctl, mc, mp, mr, pool[c.out_cur],
       c.out_prev >= 0 ? pool[c.out_prev] : nullptr, prm, g->partials, g->partials_stride, g->counters);
   TH_CHECK_LAUNCH();
@@ -636,7 +636,7 @@ static th_status tbf_launch(const Plan& P, const VecSet<float>& V, cudaStream_t 
   TH_CUDA(cudaFuncSetAttribute(k_cheb_tbf<LM, ST, LA, FI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int nblk = std::min(ntiles, sm_count());
   if (nblk > g->partials_stride) return th_fail(TH_ESTATE, "partials buffer smaller than the temporal-blocking grid");
-  k_cheb_tbf<LM, ST, LA, FI><<<nblk, dim3(TB_EX, TBF_EY), smem, st>>>(
+  th_launch(k_cheb_tbf<LM, ST, LA, FI>, nblk, dim3(TB_EX, TBF_EY), smem, st, 
       P.d, ntx, ntiles, c.in_prev >= 0 ? 1 : 0, g->ctl, mc, mp, mr, mx, my, mz, g->invd32, pool[c.out_cur],
       c.out_prev >= 0 ? pool[c.out_prev] : nullptr, prm, g->partials, g->partials_stride, g->counters);
   TH_CHECK_LAUNCH();
@@ -711,7 +711,7 @@ static th_status enq_cheb_tail(const Plan& P, const VecSet<TV>& V, const TC* gx,
       if (P.v4) {
 #define TH_CHEB4(SC, LA)                                                                                     \
   TH_UNI(P.uni && tc_f32,                                                                                    \
-         k_cheb_v4<TC, SC, LA, U><<<P.gb4, P.tb4, 0, st>>>(P.d, P.zc, g->ctl, gx, gy, gz, g->tab, V.r, zprev, \
+         th_launch(k_cheb_v4<TC, SC, LA, U>, P.gb4, P.tb4, 0, st, P.d, P.zc, g->ctl, gx, gy, gz, g->tab, V.r, zprev, \
                                                            zcur, znext, c1, c2, g->partials,                  \
                                                            g->partials_stride, g->counters))
         if (P.scaled) {
@@ -726,7 +726,7 @@ static th_status enq_cheb_tail(const Plan& P, const VecSet<TV>& V, const TC* gx,
     }
     if constexpr (sizeof(TV) == 8) {  // plain FP64 path: expanded form with the stored diagonal
 #define TH_CHEB64(SC, LA)                                                                                    \
-  k_cheb64x<SC, LA><<<P.gb, P.tb, 0, st>>>(P.d, g->ctl, g->f64, g->dg64, V.r, zprev, zcur, znext, V.invd, c1, c2, \
+  th_launch(k_cheb64x<SC, LA>, P.gb, P.tb, 0, st, P.d, g->ctl, g->f64, g->dg64, V.r, zprev, zcur, znext, V.invd, c1, c2, \
                                            g->partials, g->partials_stride, g->counters)
       if (P.scaled) {
         if (last) TH_CHEB64(true, true); else TH_CHEB64(true, false);
@@ -738,7 +738,7 @@ static th_status enq_cheb_tail(const Plan& P, const VecSet<TV>& V, const TC* gx,
       continue;
     }
 #define TH_CHEB(SC, LA)                                                                                      \
-  k_cheb<TV, TC, SC, LA><<<P.gb, P.tb, 0, st>>>(P.d, g->ctl, gx, gy, gz, g->tab, V.r, zprev, zcur, znext, \
+  th_launch(k_cheb<TV, TC, SC, LA>, P.gb, P.tb, 0, st, P.d, g->ctl, gx, gy, gz, g->tab, V.r, zprev, zcur, znext, \
                                                 V.invd, c1, c2, g->partials, g->partials_stride, g->counters)
     if (P.scaled) {
       if (last) TH_CHEB(true, true); else TH_CHEB(true, false);
@@ -771,7 +771,7 @@ static th_status enq_precond_tail(const Plan& P, const VecSet<TV>& V, cudaStream
     return th_fail(TH_EINVAL, "the multigrid preconditioner runs in FP32");
   }
   if (P.pc == TH_PC_ZLINE) {
-    k_zline<TV><<<P.gcol, P.tb, 0, st>>>(P.d, g->ctl, g->f32.gz, g->zl_m, g->zl_c, V.r, V.zc[0], g->partials,
+    th_launch(k_zline<TV>, P.gcol, P.tb, 0, st, P.d, g->ctl, g->f32.gz, g->zl_m, g->zl_c, V.r, V.zc[0], g->partials,
                                          g->partials_stride, g->counters);
     TH_CHECK_LAUNCH();
   }
@@ -785,14 +785,14 @@ static th_status enq_iteration(const Plan& P, const VecSet<TV>& V, cudaStream_t 
   thermal_grid* g = P.g;
   TV* zf = z_final(P, V);
   if constexpr (sizeof(TV) == 8) {
-    k_spmv_dot64x<<<P.gb, P.tb, 0, st>>>(P.d, g->ctl, g->f64, g->dg64, zf, V.p[parity], V.p[1 - parity], V.mu,
+    th_launch(k_spmv_dot64x<>, P.gb, P.tb, 0, st, P.d, g->ctl, g->f64, g->dg64, zf, V.p[parity], V.p[1 - parity], V.mu,
                                          g->partials, g->partials_stride, g->counters);
   } else if (P.v4) {
-    TH_UNI(P.uni, k_spmv_dot_v4<U><<<P.nbs4, P.tb4, 0, st>>>(P.d, P.zc, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz,
+    TH_UNI(P.uni, th_launch(k_spmv_dot_v4<U>, P.nbs4, P.tb4, 0, st, P.d, P.zc, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz,
                                                            g->tab, zf, V.p[parity], V.p[1 - parity], V.mu,
                                                            g->partials, g->partials_stride, g->counters));
   } else {
-    k_spmv_dot<float, float><<<P.gb, P.tb, 0, st>>>(P.d, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz, g->tab, zf,
+    th_launch(k_spmv_dot<float, float>, P.gb, P.tb, 0, st, P.d, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz, g->tab, zf,
                                                     V.p[parity], V.p[1 - parity], V.mu, g->partials,
                                                     g->partials_stride, g->counters);
   }
@@ -813,13 +813,13 @@ static void launch_residual_v4(const Plan& P, cudaStream_t st, const float* nh, 
   thermal_grid* g = P.g;
   const TP* const* pt = (const TP* const*)g->dev_ptrs;
   if (!uni) {
-    k_residual_df_v4<TP, -1, false><<<P.nbf4, P.tb4, 0, st>>>(P.d, P.zc, g->ctl, g->tab, g->f32, g->f32lo, g->th_hi,
+    th_launch(k_residual_df_v4<TP, -1, false>, P.nbf4, P.tb4, 0, st, P.d, P.zc, g->ctl, g->tab, g->f32, g->f32lo, g->th_hi,
                                                               g->th_lo, pt, nh, nl, g->r32, count_outer, ri,
                                                               g->partials, g->partials_stride, g->counters);
     return;
   }
 #define TH_RES4(ZI)                                                                                           \
-  k_residual_df_v4<TP, ZI, true><<<P.nbq4, P.tb4, 0, st>>>(P.d, P.zc, g->ctl, g->tab, g->f32, g->f32lo, g->th_hi, \
+  th_launch(k_residual_df_v4<TP, ZI, true>, P.nbq4, P.tb4, 0, st, P.d, P.zc, g->ctl, g->tab, g->f32, g->f32lo, g->th_hi, \
                                                           g->th_lo, pt, nh, nl, g->r32, count_outer, ri,        \
                                                           g->partials, g->partials_stride, g->counters)
   switch (zi) {
@@ -857,11 +857,11 @@ static th_status enq_residual(const Plan& P, cudaStream_t st, int mode, int coun
       return TH_OK;
     }
     if (P.pdtype == TH_F32)
-      TH_UNI(P.uni, k_residual_df<float, U><<<P.gb, P.tb, 0, st>>>(
+      TH_UNI(P.uni, th_launch(k_residual_df<float, U>, P.gb, P.tb, 0, st, 
                         P.d, g->ctl, g->f32, g->f32lo, g->tab, g->th_hi, g->th_lo, (const float* const*)g->dev_ptrs,
                         nh, nl, g->r32, count_outer, g->partials, g->partials_stride, g->counters));
     else
-      TH_UNI(P.uni, k_residual_df<double, U><<<P.gb, P.tb, 0, st>>>(
+      TH_UNI(P.uni, th_launch(k_residual_df<double, U>, P.gb, P.tb, 0, st, 
                         P.d, g->ctl, g->f32, g->f32lo, g->tab, g->th_hi, g->th_lo,
                         (const double* const*)g->dev_ptrs, nh, nl, g->r32, count_outer, g->partials,
                         g->partials_stride, g->counters));
@@ -871,7 +871,7 @@ static th_status enq_residual(const Plan& P, cudaStream_t st, int mode, int coun
   const double* th = g->theta[0];
   const double* thn = P.transient ? g->theta_n : nullptr;
 #define TH_RES(TP, TR, RP)                                                                                     \
-  k_residual<TP, TR><<<P.gb, P.tb, 0, st>>>(P.d, g->ctl, g->f64, g->tab, th, (const TP*)nullptr,             \
+  th_launch(k_residual<TP, TR>, P.gb, P.tb, 0, st, P.d, g->ctl, g->f64, g->tab, th, (const TP*)nullptr,             \
                                             (const TP* const*)g->dev_ptrs, thn, RP, mode, count_outer,         \
                                             g->partials, g->partials_stride, g->counters)
   if (P.pdtype == TH_F32) {
@@ -885,7 +885,7 @@ static th_status enq_residual(const Plan& P, cudaStream_t st, int mode, int coun
 }
 
 static th_status enq_cond(cudaStream_t st, cudaGraphConditionalHandle h, const Ctl* ctl, int which) {
-  k_cond<<<1, 1, 0, st>>>(h, ctl, which);
+  th_launch(k_cond, 1, 1, 0, st, h, ctl, which);
   TH_CHECK_LAUNCH();
   return TH_OK;
 }
@@ -985,9 +985,9 @@ struct Pieces {
   }
   th_status outer_close(cudaStream_t st) {  // theta += ||r|| d ; r = b - A theta
     if (P.v4)
-      k_theta_axpy_df_v4<<<P.nbu4, 256, 0, st>>>(P.d.n / 4, P.g->ctl, P.g->th_hi, P.g->th_lo, P.g->d32);
+      th_launch(k_theta_axpy_df_v4, P.nbu4, 256, 0, st, P.d.n / 4, P.g->ctl, P.g->th_hi, P.g->th_lo, P.g->d32);
     else
-      k_theta_axpy_df<<<nb1(P.d.n), 256, 0, st>>>(P.d.n, P.g->ctl, P.g->th_hi, P.g->th_lo, P.g->d32);
+      th_launch(k_theta_axpy_df, nb1(P.d.n), 256, 0, st, P.d.n, P.g->ctl, P.g->th_hi, P.g->th_lo, P.g->d32);
     TH_CHECK_LAUNCH();
     return enq_residual(P, st, 0, 1, false);
   }
@@ -1031,9 +1031,9 @@ static th_status enq_prepare(const Plan& P, cudaStream_t st, const double* T, do
   TH_CHECK_LAUNCH();
   if (P.extrap) {  // no history yet: theta_{n-1} = theta_n (the first step starts from T_0)
     if (theta64(P))
-      k_copy64<<<nb1(n), 256, 0, st>>>(n, g->theta[0], g->thm64);
+      th_launch(k_copy64, nb1(n), 256, 0, st, n, g->theta[0], g->thm64);
     else
-      k_copy_df<<<nb1(n), 256, 0, st>>>(n, g->th_hi, g->th_lo, g->thm_hi, g->thm_lo);
+      th_launch(k_copy_df, nb1(n), 256, 0, st, n, g->th_hi, g->th_lo, g->thm_hi, g->thm_lo);
     TH_CHECK_LAUNCH();
   }
   return TH_OK;
@@ -1053,25 +1053,25 @@ static th_status enq_step_copy(const Plan& P, cudaStream_t st) {
   const long long n = P.d.n;
   if (P.extrap) {
     if (theta64(P))
-      k_step_extrap64<<<nb1(n), 256, 0, st>>>(n, g->theta[0], g->theta_n, g->thm64);
+      th_launch(k_step_extrap64, nb1(n), 256, 0, st, n, g->theta[0], g->theta_n, g->thm64);
     else
       if (P.extrap_order == 3)
-        k_step_extrapq_df_v4<3><<<P.nbu4, 256, 0, st>>>(n / 4, g->ctl, g->th_hi, g->th_lo, g->thm_hi, g->thm_lo,
+        th_launch(k_step_extrapq_df_v4<3>, P.nbu4, 256, 0, st, n / 4, g->ctl, g->th_hi, g->th_lo, g->thm_hi, g->thm_lo,
                                                         g->thm2_hi, g->thm2_lo, g->thm3_hi, g->thm3_lo);
       else if (P.extrap_order == 2)
-        k_step_extrapq_df_v4<2><<<P.nbu4, 256, 0, st>>>(n / 4, g->ctl, g->th_hi, g->th_lo, g->thm_hi, g->thm_lo,
+        th_launch(k_step_extrapq_df_v4<2>, P.nbu4, 256, 0, st, n / 4, g->ctl, g->th_hi, g->th_lo, g->thm_hi, g->thm_lo,
                                                         g->thm2_hi, g->thm2_lo, nullptr, nullptr);
       else if (P.v4)
-        k_step_extrap_df_v4<<<P.nbu4, 256, 0, st>>>(n / 4, g->th_hi, g->th_lo, g->thm_hi, g->thm_lo);
+        th_launch(k_step_extrap_df_v4, P.nbu4, 256, 0, st, n / 4, g->th_hi, g->th_lo, g->thm_hi, g->thm_lo);
       else
-        k_step_extrap_df<<<nb1(n), 256, 0, st>>>(n, g->th_hi, g->th_lo, g->thm_hi, g->thm_lo);
+        th_launch(k_step_extrap_df, nb1(n), 256, 0, st, n, g->th_hi, g->th_lo, g->thm_hi, g->thm_lo);
     TH_CHECK_LAUNCH();
     return TH_OK;
   }
   if (theta64(P))
-    k_copy64<<<nb1(n), 256, 0, st>>>(n, g->theta[0], g->theta_n);
+    th_launch(k_copy64, nb1(n), 256, 0, st, n, g->theta[0], g->theta_n);
   else
-    k_copy_df<<<nb1(n), 256, 0, st>>>(n, g->th_hi, g->th_lo, g->thn_hi, g->thn_lo);
+    th_launch(k_copy_df, nb1(n), 256, 0, st, n, g->th_hi, g->th_lo, g->thn_hi, g->thn_lo);
   TH_CHECK_LAUNCH();
   return TH_OK;
 }
@@ -1109,8 +1109,14 @@ void graph_cache_free(GraphCache* c) {
   delete c;
 }
 
+thread_local int th_capturing = 0;
+
 template <class F>
 static th_status capture_body(cudaGraph_t body, cudaStream_t cs, F&& fill) {
+  struct Scope {
+    Scope() { ++th_capturing; }
+    ~Scope() { --th_capturing; }
+  } scope;
   TH_CUDA(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
   th_status st = fill(cs);
   cudaGraph_t out = nullptr;
@@ -1242,10 +1248,10 @@ static th_status build_graph(const Plan& P, int kind, const CtlInit& ci, GraphEn
       TH_TRY(begin_while(s0, ctl, 2, &bs, &hs));
       TH_TRY(capture_body(bs, gc->cs[1], [&](cudaStream_t sb) -> th_status {
         TH_TRY(enq_step_copy(P, sb));
-        k_step_begin<<<1, 1, 0, sb>>>(ctl);
+        th_launch(k_step_begin, 1, 1, 0, sb, ctl);
         TH_CHECK_LAUNCH();
         TH_TRY(emit_solve(P, gc, 1));
-        k_step_end<<<1, 1, 0, sb>>>(ctl);
+        th_launch(k_step_end, 1, 1, 0, sb, ctl);
         TH_CHECK_LAUNCH();
         return enq_cond(sb, hs, ctl, 2);
       }));
@@ -1491,10 +1497,10 @@ th_status solver_drive(thermal_grid* g, int kind, double dt, const void* const* 
       Ctl h;
       for (int step = 0; step < n_steps; ++step) {
         TH_TRY(enq_step_copy(P, s));
-        k_step_begin<<<1, 1, 0, s>>>(g->ctl);
+        th_launch(k_step_begin, 1, 1, 0, s, g->ctl);
         TH_CHECK_LAUNCH();
         TH_TRY(polled_solve(P, s));
-        k_step_end<<<1, 1, 0, s>>>(g->ctl);
+        th_launch(k_step_end, 1, 1, 0, s, g->ctl);
         TH_CHECK_LAUNCH();
         TH_TRY(poll(g, s, &h));
         if (h.status == TH_ECUDA || h.status == TH_EBREAKDOWN || h.status == TH_ENONFINITE) break;
@@ -1502,7 +1508,7 @@ th_status solver_drive(thermal_grid* g, int kind, double dt, const void* const* 
     } else {
       TH_TRY(polled_solve(P, s));
       if (kind == KIND_STEP) {
-        k_step_end<<<1, 1, 0, s>>>(g->ctl);
+        th_launch(k_step_end, 1, 1, 0, s, g->ctl);
         TH_CHECK_LAUNCH();
       }
     }
@@ -1694,49 +1700,49 @@ extern "C" th_status thermal_kernel_time(thermal_grid* g, int kernel, int reps, 
         break;
       case 1:
         if (P.v4) {
-          TH_UNI(uni, k_cheb_v4<float, true, false, U><<<P.gb4, P.tb4, 0, s>>>(
+          TH_UNI(uni, th_launch(k_cheb_v4<float, true, false, U>, P.gb4, P.tb4, 0, s, 
                           P.d, P.zc, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz, g->tab, V.r, V.zc[0], V.zc[1], V.zc[2],
                           c1, c2, g->partials, g->partials_stride, g->counters));
           break;
         }
-        k_cheb<float, float, true, false><<<P.gb, P.tb, 0, s>>>(P.d, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz, g->tab,
+        th_launch(k_cheb<float, float, true, false>, P.gb, P.tb, 0, s, P.d, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz, g->tab,
                                                                 V.r, V.zc[0], V.zc[1], V.zc[2], V.invd, c1, c2,
                                                                 g->partials, g->partials_stride, g->counters);
         break;
       case 2:
         if (P.v4) {
-          k_cheb_v4<__nv_bfloat16, true, false, false><<<P.gb4, P.tb4, 0, s>>>(
+          th_launch(k_cheb_v4<__nv_bfloat16, true, false, false>, P.gb4, P.tb4, 0, s, 
               P.d, P.zc, g->ctl, g->f16.gx, g->f16.gy, g->f16.gz, g->tab, V.r, V.zc[0], V.zc[1], V.zc[2], c1, c2,
               g->partials, g->partials_stride, g->counters);
           break;
         }
-        k_cheb<float, __nv_bfloat16, true, false><<<P.gb, P.tb, 0, s>>>(
+        th_launch(k_cheb<float, __nv_bfloat16, true, false>, P.gb, P.tb, 0, s, 
             P.d, g->ctl, g->f16.gx, g->f16.gy, g->f16.gz, g->tab, V.r, V.zc[0], V.zc[1], V.zc[2], V.invd, c1, c2,
             g->partials, g->partials_stride, g->counters);
         break;
       case 3:
         if (P.v4) {
-          TH_UNI(uni, k_spmv_dot_v4<U><<<P.nbs4, P.tb4, 0, s>>>(P.d, P.zc, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz,
+          TH_UNI(uni, th_launch(k_spmv_dot_v4<U>, P.nbs4, P.tb4, 0, s, P.d, P.zc, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz,
                                                               g->tab, V.zc[0], V.p[0], V.p[1], V.mu, g->partials,
                                                               g->partials_stride, g->counters));
           break;
         }
-        k_spmv_dot<float, float><<<P.gb, P.tb, 0, s>>>(P.d, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz, g->tab,
+        th_launch(k_spmv_dot<float, float>, P.gb, P.tb, 0, s, P.d, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz, g->tab,
                                                        V.zc[0], V.p[0], V.p[1], V.mu, g->partials,
                                                        g->partials_stride, g->counters);
         break;
       case 4:
         if (P.v4) {
-          TH_UNI(uni, k_update_v4<false, 1, U><<<P.nbr4, 256, 0, s>>>(P.d.n / 4, g->ctl, V.x, V.p[1], V.r, V.mu,
+          TH_UNI(uni, th_launch(k_update_v4<false, 1, U>, P.nbr4, 256, 0, s, P.d.n / 4, g->ctl, V.x, V.p[1], V.r, V.mu,
                                                                      V.invd, V.zc[0], 1.0f, 1, 1, 0, g->partials,
                                                                      g->partials_stride, g->counters, P.d, g->tab));
           break;
         }
-        k_update<float, false, 1><<<P.gb, P.tb, 0, s>>>(P.d, g->ctl, V.x, V.p[1], V.r, V.mu, V.invd, V.zc[0], 1.0f,
+        th_launch(k_update<float, false, 1>, P.gb, P.tb, 0, s, P.d, g->ctl, V.x, V.p[1], V.r, V.mu, V.invd, V.zc[0], 1.0f,
                                                         1, 1, 0, g->partials, g->partials_stride, g->counters);
         break;
       case 5:
-        k_residual<float, float><<<P.gb, P.tb, 0, s>>>(P.d, g->ctl, g->f64, g->tab, g->theta[0], nullptr,
+        th_launch(k_residual<float, float>, P.gb, P.tb, 0, s, P.d, g->ctl, g->f64, g->tab, g->theta[0], nullptr,
                                                        (const float* const*)g->dev_ptrs,
                                                        P.transient ? g->theta_n : nullptr, g->r32, 2, 0,
                                                        g->partials, g->partials_stride, g->counters);
@@ -1745,7 +1751,7 @@ extern "C" th_status thermal_kernel_time(thermal_grid* g, int kernel, int reps, 
         k_apply64x<<<P.gb, P.tb, 0, s>>>(P.d, g->f64, g->dg64, g->zc64[0], g->zc64[1]);
         break;
       case 7:
-        k_cheb64x<true, false><<<P.gb, P.tb, 0, s>>>(P.d, g->ctl, g->f64, g->dg64, W.r, W.zc[0], W.zc[1], W.zc[2],
+        th_launch(k_cheb64x<true, false>, P.gb, P.tb, 0, s, P.d, g->ctl, g->f64, g->dg64, W.r, W.zc[0], W.zc[1], W.zc[2],
                                                      W.invd, 0.5, 0.5, g->partials, g->partials_stride, g->counters);
         break;
       default:
@@ -1754,7 +1760,7 @@ extern "C" th_status thermal_kernel_time(thermal_grid* g, int kernel, int reps, 
                                     -1, ResidInit{}, uni);
           break;
         }
-        TH_UNI(uni, k_residual_df<float, U><<<P.gb, P.tb, 0, s>>>(
+        TH_UNI(uni, th_launch(k_residual_df<float, U>, P.gb, P.tb, 0, s, 
                         P.d, g->ctl, g->f32, g->f32lo, g->tab, g->th_hi, g->th_lo, (const float* const*)g->dev_ptrs,
                         P.transient ? g->thn_hi : nullptr, P.transient ? g->thn_lo : nullptr, g->r32, 0,
                         g->partials, g->partials_stride, g->counters));
