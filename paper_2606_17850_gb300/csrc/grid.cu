@@ -302,6 +302,7 @@ thermal_grid::~thermal_grid() {
   if (ctl_host) cudaFreeHost(ctl_host);
   if (stage_p) cudaFree(stage_p);
   dfree(stage_T);
+  if (oc_sync) cudaFree(oc_sync);
   if (dev_ptrs) cudaFree((void*)dev_ptrs);
 }
 

@@ -159,6 +159,7 @@ struct thermal_grid {
   int dev_ptrs_n = 0;
 
   GraphCache* graphs = nullptr;
+  void* oc_sync = nullptr;  // exchange words of the on-chip inner PCG
   int zc_tuned = 0;  // layers per thread in the vectorised kernels (autotuned)
 
   ~thermal_grid();
@@ -213,5 +214,23 @@ void graph_cache_free(GraphCache* c);
 // Lanczos interval and the Chebyshev three-term coefficients (c1[m], c2[m], m < k).
 th_status solver_cheb_coeffs(thermal_grid* g, double dt, const thermal_solve_opts* o, std::vector<float>& c1,
                              std::vector<float>& c2, float* inv_theta, double* lmin, double* lmax, cudaStream_t s);
+int device_sms();
+// pcg_oc.cu: the whole FP32 inner PCG with the Chebyshev preconditioner (solve = 1: on
+// r, the correction in d32), or one application of it (solve = 0: z = M^-1 r), as one
+// cooperative launch over tiles that stay on chip; layer-uniform grids whose tiles fit
+// the SMs (oc_shape's rows > 0).
+struct OCShape { int rows, halo; };
+struct OCRun {
+  OCShape shape;
+  int solve, k;
+  const float* r;
+  float* z;
+  const double *c1, *c2;  // three-term coefficients, index m < k
+  double inv_theta;
+  int expire_test;
+};
+OCShape oc_shape(int nx, int ny, int L, int k);
+th_status oc_prepare(thermal_grid* g, cudaStream_t s);
+th_status oc_run(thermal_grid* g, const OCRun& o, cudaStream_t s);
 // FP32 / BF16-coefficient y = A x through the vectorised kernel; TH_EINVAL when nx % 4 != 0.
 th_status solver_apply_f32(thermal_grid* g, bool bf16, const float* x, float* y, cudaStream_t s);

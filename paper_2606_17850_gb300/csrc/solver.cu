@@ -54,6 +54,8 @@ struct Plan {
   // pool of four FP32 buffers {zc0, zc1, zc2, mu} (indices 0..3)
   struct Chunk { int steps, m0, in_cur, in_prev, out_cur, out_prev; };
   bool fused = false;  // temporal blocking active
+  bool oc = false;     // inner PCG on chip (pcg_oc.cu)
+  OCShape oc_tile{0, 0};
   int tb_lmax = 8;  // layer capacity of the fused kernel (8: 32 x 32 tiles, 12: 32 x 24)
   std::vector<Chunk> chunks;
   int zfin = -1;  // pool index of the preconditioned vector (-1: the per-step rule)
@@ -376,10 +378,20 @@ static th_status make_plan(thermal_grid* g, double dt, const thermal_solve_opts*
     cheb_coeffs(P.lmin, P.lmax, P.k, P.c1, P.c2, &P.inv_theta);
     P.pc_spmv = P.k - 1;
     const int fuse = o->cheb_fuse == 0 ? TB_H : o->cheb_fuse;
+    // a grid whose tiles fit the SMs keeps the inner PCG on chip (any nx); an explicit
+    // cheb_fuse asks for the tile kernels
+    if (P.prec != TH_PREC_FP64 && !P.ad && P.scaled && P.uni && o->cheb_fuse == 0) {
+      P.oc_tile = oc_shape(g->nx, g->ny, g->L, P.k);
+      P.oc = P.oc_tile.rows > 0;
+    }
     // fused chunks exist for the Jacobi-scaled form (the default); the unscaled
     // polynomial of the paper runs one step per launch
     // (per-face grids: FP32 faces, so not the BF16-coefficient precision)
-    if (P.prec != TH_PREC_FP64 && !P.ad && P.v4 && P.scaled && fuse > 1 && P.k > 1 &&
+    if (P.oc) {
+      TH_TRY(oc_prepare(g, s));
+      P.fused = true;
+      P.zfin = 0;
+    } else if (P.prec != TH_PREC_FP64 && !P.ad && P.v4 && P.scaled && fuse > 1 && P.k > 1 &&
         (P.uni || P.prec == TH_PREC_MIXED_IR)) {
       // register columns: layer table up to 8 layers with 32 x 32 threads, up to 12
       // with 32 x 24; per-face arrays up to 8 layers with 32 x 24
@@ -492,7 +504,10 @@ static th_status enq_update(const Plan& P, const VecSet<TV>& V, cudaStream_t st,
   switch (P.pc) {
     case TH_PC_NONE: TH_UPD(0); break;
     case TH_PC_JACOBI: TH_UPD(1); break;
-    case TH_PC_CHEB: TH_UPD(2); break;
+    case TH_PC_CHEB:
+      if (P.oc) TH_UPD(0);
+      else TH_UPD(2);
+      break;
     default: TH_UPD(3); break;
   }
 #undef TH_UPD
@@ -548,6 +563,8 @@ static int sm_count() {
   }
   return n[dev];
 }
+
+int device_sms() { return sm_count(); }
 
 template <int LM, int EY, int ST, bool SC, bool LA, bool FI>
 static th_status tb_launch(const Plan& P, const VecSet<float>& V, cudaStream_t st, const Plan::Chunk& c) {
@@ -682,6 +699,12 @@ static th_status tb_chunk(const Plan& P, const VecSet<float>& V, cudaStream_t st
   return last ? tb_steps<LM, EY, true, true, false>(P, V, st, c) : tb_steps<LM, EY, true, false, false>(P, V, st, c);
 }
 
+// the whole inner solve (solve = 1) or one application of the polynomial, on chip
+static th_status oc_enqueue(const Plan& P, cudaStream_t st, int solve, const float* r, float* z) {
+  const OCRun o{P.oc_tile, solve, P.k, r, z, P.c1.data(), P.c2.data(), P.inv_theta, P.expire_test};
+  return oc_run(P.g, o, st);
+}
+
 static th_status tb_chain(const Plan& P, const VecSet<float>& V, cudaStream_t st) {
   for (size_t ci = 0; ci < P.chunks.size(); ++ci) {
     const bool last = (ci + 1 == P.chunks.size());
@@ -698,6 +721,7 @@ static th_status enq_cheb_tail(const Plan& P, const VecSet<TV>& V, const TC* gx,
                                cudaStream_t st) {
   thermal_grid* g = P.g;
   if constexpr (sizeof(TV) == 4) {
+    if (P.oc) return oc_enqueue(P, st, 0, V.r, V.zc[0]);
     if (P.fused) return tb_chain(P, V, st);
   }
   for (int m = 1; m < P.k; ++m) {
@@ -976,6 +1000,7 @@ struct Pieces {
   th_status inner_init(cudaStream_t st) {
     VecSet<float> V = vec32(P.g);
     if (!P.fused_init) TH_TRY((enq_update<float, true>(P, V, st, 0, 1, 1)));
+    if (P.oc) return oc_enqueue(P, st, 1, P.g->r32, nullptr);  // the whole inner solve
     return enq_precond_tail<float>(P, V, st);
   }
   th_status inner_pair(cudaStream_t st) {
@@ -1202,13 +1227,15 @@ static th_status emit_solve(const Plan& P, GraphCache* gc, int lvl) {
   TH_TRY(begin_while(s, ctl, 1, &bo, &ho));
   return capture_body(bo, gc->cs[lvl + 1], [&](cudaStream_t sb) -> th_status {
     TH_TRY(pcs.inner_init(sb));
-    cudaGraph_t bi;
-    cudaGraphConditionalHandle hi;
-    TH_TRY(begin_while(sb, ctl, 0, &bi, &hi));
-    TH_TRY(capture_body(bi, gc->cs[lvl + 2], [&](cudaStream_t sc) -> th_status {
-      TH_TRY(pcs.inner_pair(sc));
-      return enq_cond(sc, hi, ctl, 0);
-    }));
+    if (!P.oc) {
+      cudaGraph_t bi;
+      cudaGraphConditionalHandle hi;
+      TH_TRY(begin_while(sb, ctl, 0, &bi, &hi));
+      TH_TRY(capture_body(bi, gc->cs[lvl + 2], [&](cudaStream_t sc) -> th_status {
+        TH_TRY(pcs.inner_pair(sc));
+        return enq_cond(sc, hi, ctl, 0);
+      }));
+    }
     TH_TRY(pcs.outer_close(sb));
     return enq_cond(sb, ho, ctl, 1);
   });
@@ -1325,9 +1352,9 @@ static th_status polled_solve(const Plan& P, cudaStream_t s) {
   TH_TRY(poll(g, s, &h));
   while (!h.outer_done) {
     TH_TRY(pcs.inner_init(s));
-    TH_TRY(poll(g, s, &h));
+    if (!P.oc) TH_TRY(poll(g, s, &h));
     int chunk = 2;
-    while (!h.done) {
+    while (!P.oc && !h.done) {
       for (int c = 0; c < chunk; ++c) TH_TRY(pcs.inner_pair(s));
       TH_TRY(poll(g, s, &h));
       chunk = std::min(chunk * 2, 32);
@@ -1605,6 +1632,11 @@ extern "C" th_status thermal_precond_apply(thermal_grid* g, double dt, const the
   o.precision = (opts->precision == TH_PREC_MIXED_IR_BF16) ? TH_PREC_MIXED_IR_BF16 : TH_PREC_MIXED_IR;
   Plan P;
   TH_TRY(make_plan(g, dt, &o, TH_F32, dt > 0.0, P, s));
+  if (P.oc && (z + g->n <= r || r + g->n <= z)) {  // one launch from r to z
+    TH_TRY(oc_enqueue(P, s, 0, r, z));
+    TH_CUDA(cudaStreamSynchronize(s));
+    return TH_OK;
+  }
   const CtlInit ci = ctl_init(&o, 1, 1, 1);
   k_ctl_reset<<<1, 1, 0, s>>>(g->ctl, ci);
   TH_CHECK_LAUNCH();

@@ -1055,3 +1055,71 @@ def test_mixed_solve_chebyshev_variants(scaled, fuse, k):
     assert stats["status"] == 0
     ref = osolve.transient(nx, ny, st, [P] * 4, dt, T0)[-1]
     assert osolve.rise_relative_error(T.cpu().numpy(), ref, st.t_amb) <= 1e-6
+
+
+# ----------------------------------------------------- on-chip inner PCG (small layer-uniform grids)
+
+# (nx, ny, stack, k): nx % 4 == 0 and not (expanded / difference form), one column, one
+# tile, rows of tiles, tile counts at 1 and many, 1 to 12 layers; k - 1 below, at and above
+# multiples of the halo, and the two ends of the degree range that runs on chip
+ONCHIP = [(1, 1, "c2", 2), (5, 3, "c1", 9), (64, 64, "c1", 30), (24, 8, "l5", 5), (25, 9, "l6", 4), (130, 70, "c1", 12),
+          (131, 37, "l7", 13), (200, 160, "c2", 30), (287, 203, "c2", 17), (76, 37, "mol", 8), (63, 90, "mol", 128),
+          (288, 288, "c2", 10)]
+
+
+@pytest.mark.parametrize("nx,ny,mk,k", ONCHIP)
+def test_onchip_chebyshev_equals_stepwise(nx, ny, mk, k):
+    """One cooperative launch for the whole polynomial against one launch per step."""
+    st = STACKS[mk]()
+    g = grid_of(nx, ny, st)
+    r = cuda(ti.random_vector(nx * ny * st.L, 5).astype(np.float32))
+    for dt in (0.0, 1e-4):
+        z1 = g.precond(r, dt, precond="cheb", cheb_degree=k, cheb_fuse=1)
+        z0 = g.precond(r, dt, precond="cheb", cheb_degree=k)
+        # the bound of the fused chunks (expanded form, see above)
+        assert (z0 - z1).abs().max().item() <= max(1e-6, 2.5e-7 * k) * z1.abs().max().item(), dt
+        assert torch.equal(z0, g.precond(r, dt, precond="cheb", cheb_degree=k))  # deterministic
+
+
+@pytest.mark.parametrize("graph", [0, 1])
+@pytest.mark.parametrize("nx,ny,mk,k", [(5, 3, "c1", 4), (64, 64, "c1", 30), (131, 37, "l7", 13), (76, 37, "mol", 8),
+                                        (200, 160, "c2", 9)])
+def test_onchip_solve_matches_stepwise_solve(nx, ny, mk, k, graph):
+    """Steady solve and time steps with the inner PCG on chip against the per-step kernels:
+    the same system to the same tolerance."""
+    st = STACKS[mk]()
+    g = grid_of(nx, ny, st)
+    P = cuda(ti.power_cells(st, nx, ny, [ti.density_uniform_hotspots(nx, ny, s + 1) for s, _ in
+                                         enumerate(st.power_layers())], np.float32))
+    o = dict(precond="cheb", cheb_degree=k, tol_rel=1e-9, use_graph=graph)
+    (T0, s0), (T1, s1) = g.solve_steady(P, **o), g.solve_steady(P, cheb_fuse=1, **o)
+    rise = (T1 - st.t_amb).abs().max().item()
+    assert s0["rel_res"] <= 1e-9 and s1["rel_res"] <= 1e-9
+    assert (T0 - T1).abs().max().item() <= 1e-6 * rise
+    t0 = torch.full((g.n,), st.t_amb, dtype=torch.float64, device="cuda")
+    t1 = t0.clone()
+    g.run_transient([P], 2, 5, 1e-4, t0, guess=1, **o)
+    g.run_transient([P], 2, 5, 1e-4, t1, guess=1, cheb_fuse=1, **o)
+    assert (t0 - t1).abs().max().item() <= 1e-6 * (t1 - st.t_amb).abs().max().item()
+
+
+@pytest.mark.parametrize("graph", [0, 1])
+def test_onchip_wait_expiry_and_limits(graph):
+    """A wait that runs out (2 ms, a number nothing writes) gives TH_ECUDA and the next
+    solve on the grid is right; an inner iteration limit ends the inner solve."""
+    from paper_2606_17850_gb300 import ThermalError
+    st = ti.stack_c2()
+    nx, ny = 77, 37
+    g = grid_of(nx, ny, st)
+    P = cuda(ti.power_cells(st, nx, ny, [ti.density_uniform_hotspots(nx, ny, 4) for _ in st.power_layers()],
+                            np.float32))
+    o = dict(precond="cheb", cheb_degree=12, use_graph=graph)
+    ref, _ = g.solve_steady(P, cheb_fuse=1, tol_rel=1e-10, **o)
+    with pytest.raises(ThermalError) as e:
+        g.solve_steady(P, test_wait_expire=1, tol_rel=1e-10, **o)
+    assert e.value.status == 3 and "timed out" in str(e.value)
+    T, s = g.solve_steady(P, tol_rel=1e-10, **o)
+    assert (T - ref).abs().max().item() <= 1e-6 * (ref - st.t_amb).abs().max().item()
+    with pytest.raises(ThermalError) as e:
+        g.solve_steady(P, tol_rel=1e-10, max_outer=2, max_inner=3, **o)
+    assert e.value.status == 4
