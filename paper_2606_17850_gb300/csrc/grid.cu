@@ -5,6 +5,7 @@
 // face is the series combination of the two half cells it joins, the top face of
 // the top layer adds h dx dy to the diagonal, and a backward-Euler step adds
 // c dx dy dz / dt.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -467,7 +468,8 @@ th_status grid_ensure_workspace(thermal_grid* g, bool need64, cudaStream_t s) {
     TH_TRY(dalloc(&g->thn_hi, n));
     TH_TRY(dalloc(&g->thn_lo, n));
     const dim3 gb = grid_blocks(g);
-    g->partials_stride = (int)(gb.x * gb.y * gb.z);
+    // one slot per block of any reducing kernel: cell blocks, or resident blocks
+    g->partials_stride = std::max((int)(gb.x * gb.y * gb.z), 8 * device_sms());
     TH_TRY(dalloc(&g->partials, (size_t)4 * g->partials_stride + 64));
     TH_TRY(dalloc(&g->counters, 64));
     TH_CUDA(cudaMemsetAsync(g->counters, 0, 64 * sizeof(unsigned), s));

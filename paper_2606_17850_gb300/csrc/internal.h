@@ -195,7 +195,6 @@ struct MGBDesc {
 // Builds (or reuses) the hierarchy of g for the steady matrix and fills *out;
 // TH_EINVAL when it has more than MG_BMAXL levels.
 th_status mg_batch_levels(thermal_grid* g, MGBDesc* out, cudaStream_t s);
-th_status mg_rz(thermal_grid* g, const float* r, const float* z, cudaStream_t s);
 dim3 grid_blocks(const thermal_grid* g);
 Dims grid_dims(const thermal_grid* g);
 bool is_device_pointer(const void* p);

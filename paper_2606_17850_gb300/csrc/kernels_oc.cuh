@@ -155,13 +155,21 @@ __device__ __forceinline__ bool oc_sum(OCShared& sh, OCWord* sync, int cap, unsi
     double tot = 0.0;
     bool ok = true;
     unsigned long long t0 = 0;
-    for (int j = t; j < nblk && ok; j += 32) {
-      OCWord w = oc_get(set + j);
-      while (ok && (unsigned)w.hi != epoch) {
-        ok = !oc_late(t0);
-        w = oc_get(set + j);
+    for (int j0 = t; j0 < nblk && ok; j0 += 32 * 5) {  // a lane reads its slots together
+      OCWord w[5];
+      bool behind = true;
+      while (behind && ok) {
+        behind = false;
+#pragma unroll
+        for (int i = 0; i < 5; ++i)
+          if (j0 + 32 * i < nblk) w[i] = oc_get(set + j0 + 32 * i);
+          else w[i] = OCWord{0ull, epoch};
+#pragma unroll
+        for (int i = 0; i < 5; ++i) behind = behind || (unsigned)w[i].hi != epoch;
+        if (behind) ok = !oc_late(t0);
       }
-      tot += __longlong_as_double((long long)w.lo);
+#pragma unroll
+      for (int i = 0; i < 5; ++i) tot += __longlong_as_double((long long)w[i].lo);
     }
     ok = __all_sync(0xffffffffu, ok);
     tot = warp_sum(tot);

@@ -24,10 +24,10 @@
 
 #include "internal.h"
 #include "mg_device.cuh"
+#include "mg_tile.cuh"
 
 namespace {
 
-constexpr float MG_OMEGA = kMGOmega;
 constexpr int MG_COARSEST = 8;
 
 __device__ __forceinline__ long long idx3(int nx, int ny, int x, int y, int z) {
@@ -103,321 +103,147 @@ __global__ void k_mg_zfactors(int nx, int ny, int L, const float* __restrict__ g
   }
 }
 
-// x_out = x + omega T^-1 (b - A x) per column (mg_smooth_column), one thread per column
-template <int LMAX, bool UNI>
-__global__ void __launch_bounds__(256) k_mg_smooth(const Ctl* ctl, MGDev v, const __grid_constant__ MGUni<LMAX> U,
-                                                   const float* __restrict__ b, const float* __restrict__ xin,
-                                                   const float* __restrict__ xc, int nxc, int nyc,
-                                                   float* __restrict__ xout, float omega) {
-  grid_dep_enter();
-  if (ld_int(&ctl->done)) return;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  if (x >= v.nx || y >= v.ny) return;
-  mg_smooth_column<LMAX, UNI>(v, U, x, y, b, xin, xc, nxc, nyc, xout, omega, false);
-}
+// ---------------------------------------------------------------- the cycle's kernels
+// A level is two passes (mg_tile.cuh): smoothing from zero + residual + restriction on the
+// way down, prolongation + smoothing on the way up, each reading its vectors once.  Levels
+// with more tiles than a cluster has blocks run them as launches of their own; the levels
+// below run, way down, coarsest solve and way up, in one launch of a single cluster whose
+// blocks meet at its hardware barrier: they are bound by the latency of a pass, not by
+// work, and a grid has four or five of them.  Measured V-cycles with r^T z, before (two
+// launches down and one up per level, r^T z apart) and now: 64^2 x 4 42 -> 18.5 us, 128^2 x
+// 8 69 -> 31, 357 x 301 x 8 168 -> 61, 512^2 x 8 126 -> 60, 1024^2 x 8 225 -> 132, 1024^2 x
+// 10 287 -> 181.  (All these levels in one cooperative grid with a barrier in memory: 84 ->
+// 108 us at 512^2; a phase there costs 5 us.)  The finest level is bound by the latency of
+// a tile's load - solve - store chain at 32 warps an SM (2.3 to 2.5 TB/s).
 
-// b_c = P^T (b - A x) (mg_restrict_tile), block (32, 8)
-template <int LMAX, bool UNI>
-__global__ void __launch_bounds__(256) k_mg_restrict(const Ctl* ctl, MGDev v, const __grid_constant__ MGUni<LMAX> U,
-                                                     const float* __restrict__ b, const float* __restrict__ x,
-                                                     int nxc, int nyc, float* __restrict__ bc) {
-  grid_dep_enter();
-  if (ld_int(&ctl->done)) return;
-  __shared__ float rowsum[8][32];
-  mg_restrict_tile<LMAX, UNI>(v, U, blockIdx.x, blockIdx.y, b, x, nxc, nyc, bc, rowsum);
-}
+// Rows of a block's grown tile, and blocks per SM that the registers allow.  Measured
+// V-cycles (us, 512^2 x 8 / 357 x 301 x 8 / 1024^2 x 8 / 1024^2 x 10): 16 rows at 2 blocks
+// 64.0 / 76.8 / 134.7 / 180.7, at 3 blocks 64.1 / 91.2 / 133.2 / 189.8; 8 rows at 4 blocks
+// 60.4 / 60.7 / 131.9 / 181.3, at 6 blocks 62.3 / 74.9 / 131.1 / 183.6.
+constexpr int MG_EY = 8;
+constexpr unsigned MG_MINB = 4;
+constexpr int MG_CLUSTER = 16;  // blocks of the cluster (8 where 16 cannot be scheduled)
 
-// ---------------------------------------------------------------- finest level, vectorised
-// Layer-uniform grids with nx % 4 == 0 and at most 8 layers: a thread owns 4
-// consecutive columns (x0 .. x0+3, x0 % 4 == 0) and moves them with 16-byte loads;
-// the two aggregates they belong to (x0/2, x0/2+1) are one 8-byte load of the
-// coarse correction.  Same arithmetic as k_mg_smooth / k_mg_restrict.
-
-__device__ __forceinline__ float4 mg_ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ float2 mg_ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
-__device__ __forceinline__ float mg_c4(const float4& v, int k) {
-  return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w));
-}
-
-// the 4 columns' iterate (x_in + P x_c) at row yy, layer z, and the scalar neighbours
-struct MGRow4 {
-  const float* xin;
-  const float* xc;
-  int nx, nxc;
-  long long pxy, pxyc;
-  __device__ __forceinline__ float4 row(int x0, int yy, int z) const {
-    if (!xin) return make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 t = mg_ld4(xin + (long long)x0 + (long long)nx * yy + pxy * z);
-    if (xc) {
-      const float2 c = mg_ld2(xc + (x0 >> 1) + (long long)nxc * (yy >> 1) + pxyc * z);
-      t.x += c.x; t.y += c.x; t.z += c.y; t.w += c.y;
-    }
-    return t;
-  }
-  __device__ __forceinline__ float one(int xx, int yy, int z) const {
-    if (!xin) return 0.f;
-    float t = xin[(long long)xx + (long long)nx * yy + pxy * z];
-    if (xc) t += xc[(xx >> 1) + (long long)nxc * (yy >> 1) + pxyc * z];
-    return t;
-  }
+template <int LMAX>
+struct MGCLev {
+  int nx, ny, uni, pad;
+  const float *gx, *gy, *gz, *s, *m, *w;
+  float *x, *xt, *b;
+  MGUni<LMAX> t;
 };
 
 template <int LMAX>
-__global__ void __launch_bounds__(256, 2) k_mg_smooth4(const Ctl* ctl, int nx, int ny, int L,
-                                                       const __grid_constant__ MGUni<LMAX> U,
-                                                       const float* __restrict__ b, const float* __restrict__ xin,
-                                                       const float* __restrict__ xc, int nxc, int nyc,
-                                                       float* __restrict__ xout, float omega) {
-  grid_dep_enter();
-  if (ld_int(&ctl->done)) return;
-  const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  if (x0 >= nx || y >= ny) return;
-  const long long pxy = (long long)nx * ny;
-  const MGRow4 X{xin, xc, nx, nxc, pxy, (long long)nxc * nyc};
-  const bool hasL = x0 > 0, hasR = x0 + 4 < nx, hasD = y > 0, hasU = y + 1 < ny;
-  const int nyf = (int)hasU + (int)hasD;
-  // boundary case of each of the 4 columns (only the outer two can miss an x neighbour)
-  const int cs0 = (1 + (int)hasL) + 3 * nyf, cs3 = (1 + (int)hasR) + 3 * nyf, csm = 2 + 3 * nyf;
-  float xv[4][LMAX], dp[4][LMAX];
-  float4 xb = make_float4(0.f, 0.f, 0.f, 0.f);
-  float4 xcur = X.row(x0, y, 0);
-  float dprev[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int z = 0; z < LMAX; ++z) {
-    if (z >= L) break;
-    const long long i = (long long)x0 + (long long)nx * y + pxy * z;
-    const float4 xa = (xin && z + 1 < L) ? X.row(x0, y, z + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float4 bv = mg_ld4(b + i);
-    float4 xu = xcur, xd = xcur;
-    float xl = xcur.x, xr = xcur.w;
-    if (xin) {
-      if (hasU) xu = X.row(x0, y + 1, z);
-      if (hasD) xd = X.row(x0, y - 1, z);
-      if (hasL) xl = X.one(x0 - 1, y, z);
-      if (hasR) xr = X.one(x0 + 4, y, z);
-    }
-    const float gx = U.gx[z], gy = U.gy[z], ga = U.gz[z], gbz = z > 0 ? U.gz[z > 0 ? z - 1 : 0] : 0.f;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float xi = mg_c4(xcur, k);
-      xv[k][z] = xi;
-      float res = mg_c4(bv, k);
-      if (xin) {
-        const float right = (k == 3) ? xr : mg_c4(xcur, k + 1);
-        const float left = (k == 0) ? xl : mg_c4(xcur, k - 1);
-        float a = U.s[z] * xi;
-        if (k < 3 || hasR) a += gx * (xi - right);
-        if (k > 0 || hasL) a += gx * (xi - left);
-        if (hasU) a += gy * (xi - mg_c4(xu, k));
-        if (hasD) a += gy * (xi - mg_c4(xd, k));
-        if (z + 1 < L) a += ga * (xi - mg_c4(xa, k));
-        if (z > 0) a += gbz * (xi - mg_c4(xb, k));
-        res -= a;
-      }
-      const int c = (k == 0) ? cs0 : ((k == 3) ? cs3 : csm);
-      dprev[k] = (res + gbz * dprev[k]) * U.m[c][z];
-      dp[k][z] = dprev[k];
-    }
-    xb = xcur;
-    xcur = xa;
-  }
-  float dn[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int zz = LMAX - 1; zz >= 0; --zz) {
-    if (zz >= L) continue;
-    float o[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int c = (k == 0) ? cs0 : ((k == 3) ? cs3 : csm);
-      const float d = dp[k][zz] + U.w[c][zz] * dn[k];
-      dn[k] = d;
-      o[k] = xv[k][zz] + omega * d;
-    }
-    *reinterpret_cast<float4*>(xout + (long long)x0 + (long long)nx * y + pxy * zz) = make_float4(o[0], o[1], o[2], o[3]);
-  }
+constexpr size_t mg_xs_bytes() {
+  return sizeof(float) * LMAX * MGT_EX * MG_EY;
 }
 
-// b_c = P^T (b - A x) on the vectorised finest level: 4 fine columns give 2 aggregate
-// partial sums per layer; the y pair is summed through shared memory.  Block (32, 8).
-// The column walks its layers keeping the layer below and the current one in
-// registers (one new layer of x per step), and holds every layer's pair sums until a
-// single block barrier, so the layers' loads are not serialised by barriers.
-template <int LMAX>
-__global__ void __launch_bounds__(256) k_mg_restrict4(const Ctl* ctl, int nx, int ny, int L,
-                                                      const __grid_constant__ MGUni<LMAX> U,
-                                                      const float* __restrict__ b, const float* __restrict__ x,
-                                                      int nxc, int nyc, float* __restrict__ bc) {
+template <int LMAX, bool UNI>
+__global__ void __launch_bounds__(MGT_EX* MG_EY, LMAX <= 12 ? MG_MINB : 1)
+    k_mg_down(const Ctl* ctl, MGDev v, const __grid_constant__ MGUni<LMAX> U, const float* __restrict__ b,
+              float* __restrict__ x, int nxc, int nyc, float* __restrict__ bc) {
   grid_dep_enter();
   if (ld_int(&ctl->done)) return;
-  __shared__ float2 rowsum[LMAX][8][32];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int x0 = 4 * (blockIdx.x * 32 + tx), y = blockIdx.y * 8 + ty;
-  const bool in = x0 < nx && y < ny;
-  const long long pxy = (long long)nx * ny;
-  const bool hasL = x0 > 0, hasR = x0 + 4 < nx, hasD = y > 0, hasU = y + 1 < ny;
-  if (in) {
-    const long long i0 = (long long)x0 + (long long)nx * y;
-    float4 xbv = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 xc = mg_ld4(x + i0);
-#pragma unroll
-    for (int z = 0; z < LMAX; ++z) {
-      if (z >= L) break;
-      const long long i = i0 + pxy * z;
-      const float4 bv = mg_ld4(b + i);
-      const float4 xu = hasU ? mg_ld4(x + i + nx) : xc, xd = hasD ? mg_ld4(x + i - nx) : xc;
-      const float4 xa = (z + 1 < L) ? mg_ld4(x + i + pxy) : xc;
-      const float4 xbz = (z > 0) ? xbv : xc;
-      const float xl = hasL ? x[i - 1] : xc.x, xr = hasR ? x[i + 4] : xc.w;
-      const float gx = U.gx[z], gy = U.gy[z], ga = U.gz[z], gbz = z > 0 ? U.gz[z > 0 ? z - 1 : 0] : 0.f;
-      float r[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float xi = mg_c4(xc, k);
-        const float right = (k == 3) ? xr : mg_c4(xc, k + 1);
-        const float left = (k == 0) ? xl : mg_c4(xc, k - 1);
-        float a = U.s[z] * xi;
-        a += gx * (xi - right);  // a missing neighbour is the cell itself: difference 0
-        a += gx * (xi - left);
-        a += gy * (xi - mg_c4(xu, k));
-        a += gy * (xi - mg_c4(xd, k));
-        a += ga * (xi - mg_c4(xa, k));
-        a += gbz * (xi - mg_c4(xbz, k));
-        r[k] = mg_c4(bv, k) - a;
-      }
-      rowsum[z][ty][tx] = make_float2(r[0] + r[1], r[2] + r[3]);
-      xbv = xc;
-      xc = xa;
-    }
-  } else {
-#pragma unroll
-    for (int z = 0; z < LMAX; ++z)
-      if (z < L) rowsum[z][ty][tx] = make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  if ((ty & 1) == 0) {
-    const int X0 = x0 >> 1, Y = y >> 1;
-    if (X0 < nxc && Y < nyc) {
-#pragma unroll
-      for (int z = 0; z < LMAX; ++z) {
-        if (z >= L) break;
-        const float2 a = rowsum[z][ty][tx], c = rowsum[z][ty + 1][tx];
-        *reinterpret_cast<float2*>(bc + X0 + (long long)nxc * Y + (long long)nxc * nyc * z) =
-            make_float2(a.x + c.x, a.y + c.y);
-      }
-    }
-  }
+  extern __shared__ float mg_xs[];
+  mgt_down<LMAX, UNI, MG_EY, false>(v, U, blockIdx.x, blockIdx.y, b, x, nxc, nyc, bc, mg_xs);
 }
 
-// ---------------------------------------------------------------- coarse levels, column tiles
-// Layer-uniform coarse levels are small: their kernels are bound by memory latency,
-// not bandwidth.  A block takes 8 x 4 columns and every layer, one thread per cell:
-// each thread forms its cell's residual with one round of independent loads into
-// shared memory, then one warp runs the 32 columns' tridiagonal solves from shared
-// memory (the smoother) or the block sums its 2 x 2 aggregates (the restriction).
-// Same arithmetic as k_mg_smooth / k_mg_restrict with the level's table.
-#define MG_CT_X 8
-#define MG_CT_Y 4
-
-template <int LMAX>
-__device__ __forceinline__ float mg_ct_residual(const MGUni<LMAX>& U, int nx, int ny, int L, int x, int y, int z,
-                                                float bi, float xi, const float* __restrict__ xin,
-                                                const float* __restrict__ xc, int nxc, long long pxyc) {
-  // the iterate at a neighbour: x_in + P x_c (the coarse correction read on the fly)
-  auto val = [&](int xx, int yy, int zz) -> float {
-    float t = xin[(long long)xx + (long long)nx * ((long long)yy + (long long)ny * zz)];
-    if (xc) t += xc[(xx >> 1) + (long long)nxc * (yy >> 1) + pxyc * zz];
-    return t;
-  };
-  float a = U.s[z] * xi;
-  if (x + 1 < nx) a += U.gx[z] * (xi - val(x + 1, y, z));
-  if (x > 0) a += U.gx[z] * (xi - val(x - 1, y, z));
-  if (y + 1 < ny) a += U.gy[z] * (xi - val(x, y + 1, z));
-  if (y > 0) a += U.gy[z] * (xi - val(x, y - 1, z));
-  if (z + 1 < L) a += U.gz[z] * (xi - val(x, y, z + 1));
-  if (z > 0) a += U.gz[z > 0 ? z - 1 : 0] * (xi - val(x, y, z - 1));
-  return bi - a;
-}
-
-// x_out = x + omega T^-1 (b - A x), x = x_in (+ P x_c) or 0.  Block (32, LMAX).
-template <int LMAX>
-__global__ void __launch_bounds__(32 * LMAX) k_mg_smooth_ct(const Ctl* ctl, int nx, int ny, int L,
-                                                           const __grid_constant__ MGUni<LMAX> U,
-                                                           const float* __restrict__ b,
-                                                           const float* __restrict__ xin,
-                                                           const float* __restrict__ xc, int nxc, int nyc,
-                                                           float* __restrict__ xout, float omega) {
+// way up; on the finest level (RZ) with r^T z and beta (b is r)
+template <int LMAX, bool UNI, bool RZ>
+__global__ void __launch_bounds__(MGT_EX* MG_EY, LMAX <= 12 ? MG_MINB : 1)
+    k_mg_up(Ctl* ctl, MGDev v, const __grid_constant__ MGUni<LMAX> U, const float* __restrict__ b,
+            const float* __restrict__ xin, const float* __restrict__ xc, int nxc, int nyc, float* __restrict__ xout,
+            double* partials, int stride, unsigned* counter) {
   grid_dep_enter();
   if (ld_int(&ctl->done)) return;
-  __shared__ float sr[LMAX][32], sx[LMAX][32];
-  const int t = threadIdx.x, z = threadIdx.y;
-  const int x = blockIdx.x * MG_CT_X + (t % MG_CT_X), y = blockIdx.y * MG_CT_Y + (t / MG_CT_X);
-  const bool col = x < nx && y < ny;
-  const long long i = (long long)x + (long long)nx * ((long long)y + (long long)ny * z);
-  float res = 0.f, xi = 0.f;
-  if (col && z < L) {
-    const float bi = b[i];
-    if (xin) {
-      xi = xin[i];
-      if (xc) xi += xc[(x >> 1) + (long long)nxc * (y >> 1) + (long long)nxc * nyc * z];
-      res = mg_ct_residual<LMAX>(U, nx, ny, L, x, y, z, bi, xi, xin, xc, nxc, (long long)nxc * nyc);
-    } else {
-      res = bi;
-    }
+  extern __shared__ float mg_xs[];
+  if (!RZ) {
+    mgt_up<LMAX, UNI, MG_EY, false, RZ>(v, U, blockIdx.x, blockIdx.y, b, xin, xc, nxc, nyc, xout, mg_xs);
+    return;
   }
-  sr[z][t] = res;
-  sx[z][t] = xi;
-  __syncthreads();
-  if (z == 0 && col) {  // one warp: the 32 columns' Thomas solves
-    const int cs = (int)(x + 1 < nx) + (int)(x > 0) + 3 * ((int)(y + 1 < ny) + (int)(y > 0));
-    float dprev = 0.f;
-#pragma unroll
-    for (int zz = 0; zz < LMAX; ++zz) {
-      if (zz >= L) break;
-      const float gb = zz > 0 ? U.gz[zz > 0 ? zz - 1 : 0] : 0.f;
-      dprev = (sr[zz][t] + gb * dprev) * U.m[cs][zz];
-      sr[zz][t] = dprev;
-    }
-    float dn = 0.f;
-#pragma unroll
-    for (int zz = LMAX - 1; zz >= 0; --zz) {
-      if (zz >= L) continue;
-      const float d = sr[zz][t] + U.w[cs][zz] * dn;
-      dn = d;
-      sr[zz][t] = sx[zz][t] + omega * d;
-    }
+  // the tiles over the blocks that are resident at once, so that the reduction's tail (7 us
+  // of 19 with one tile per block at 512 x 512 x 8) is paid once per block
+  float part[1] = {0.f};
+  const int tx = (v.nx + MGT_EX - 3) / (MGT_EX - 2);
+  for (int q = blockIdx.x; q < mgt_tiles<MG_EY>(v.nx, v.ny); q += gridDim.x) {
+    part[0] += mgt_up<LMAX, UNI, MG_EY, false, RZ>(v, U, q % tx, q / tx, b, xin, xc, nxc, nyc, xout, mg_xs);
+    __syncthreads();
   }
-  __syncthreads();
-  if (col && z < L) xout[i] = sr[z][t];
+  double tot[1];
+  if (!grid_reduce<float, 1>(part, partials, stride, counter, tot)) return;
+  ctl->rz_next = tot[0];
+  ctl_set_beta(ctl);
 }
 
-// b_c = P^T (b - A x) for complete 2 x 2 aggregates (even nx, ny).  Block (32, LMAX).
+__device__ __forceinline__ void mg_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Levels k0 .. nl - 1 of one cycle by one cluster.  b0: right-hand side of level k0
+// (level 0: r); z: where level 0's result goes (k0 = 0), with r^T z and beta.
 template <int LMAX>
-__global__ void __launch_bounds__(32 * LMAX) k_mg_restrict_ct(const Ctl* ctl, int nx, int ny, int L,
-                                                             const __grid_constant__ MGUni<LMAX> U,
-                                                             const float* __restrict__ b,
-                                                             const float* __restrict__ x, int nxc, int nyc,
-                                                             float* __restrict__ bc) {
+__global__ void __launch_bounds__(MGT_EX* MG_EY, 1)
+    k_mg_levels(Ctl* ctl, const MGCLev<LMAX>* lv, int L, int k0, int nl, int nc, const float* __restrict__ cinv,
+                const float* b0, float* z, double* partials, int stride, unsigned* counter) {
   grid_dep_enter();
-  if (ld_int(&ctl->done)) return;
-  __shared__ float sr[LMAX][32];
-  const int t = threadIdx.x, z = threadIdx.y;
-  const int cx = t % MG_CT_X, cy = t / MG_CT_X;
-  const int xx = blockIdx.x * MG_CT_X + cx, yy = blockIdx.y * MG_CT_Y + cy;
-  float r = 0.f;
-  if (xx < nx && yy < ny && z < L) {
-    const long long i = (long long)xx + (long long)nx * ((long long)yy + (long long)ny * z);
-    r = mg_ct_residual<LMAX>(U, nx, ny, L, xx, yy, z, b[i], x[i], x, nullptr, 1, 0);
+  extern __shared__ float mg_xs[];
+  MGCLev<LMAX>* sl = reinterpret_cast<MGCLev<LMAX>*>(mg_xs + LMAX * MGT_EX * MG_EY);  // levels k0 ..
+  const int t = thread_linear_id();
+  {
+    const int* src = reinterpret_cast<const int*>(lv + k0);
+    int* dst = reinterpret_cast<int*>(sl);
+    for (int i = t; i < (int)(sizeof(MGCLev<LMAX>) / 4) * (nl - k0); i += MGT_EX * MG_EY) dst[i] = __ldg(src + i);
   }
-  sr[z][t] = r;
-  __syncthreads();
-  if (((cx | cy) & 1) == 0 && z < L) {
-    const int X = xx >> 1, Y = yy >> 1;
-    if (X < nxc && Y < nyc)
-      bc[(long long)X + (long long)nxc * ((long long)Y + (long long)nyc * z)] =
-          (sr[z][t] + sr[z][t + 1]) + (sr[z][t + MG_CT_X] + sr[z][t + MG_CT_X + 1]);
+  if (__syncthreads_or(t == 0 && ld_int(&ctl->done))) return;  // set by an earlier kernel: every block sees it
+  float part[1] = {0.f};
+  for (int k = k0; k + 1 < nl; ++k) {
+    const MGCLev<LMAX>& l = sl[k - k0];
+    const int nxc = (l.nx + 1) / 2, nyc = (l.ny + 1) / 2, tx = (l.nx + MGT_EX - 3) / (MGT_EX - 2);
+    const MGDev v{l.nx, l.ny, L, l.gx, l.gy, l.gz, l.s, l.m, l.w};
+    const float* b = k == k0 ? b0 : l.b;
+    float* bc = sl[k + 1 - k0].b;
+    for (int q = blockIdx.x; q < mgt_tiles<MG_EY>(l.nx, l.ny); q += gridDim.x) {
+      __syncthreads();
+      if (l.uni) mgt_down<LMAX, true, MG_EY, true>(v, l.t, q % tx, q / tx, b, l.x, nxc, nyc, bc, mg_xs);
+      else mgt_down<LMAX, false, MG_EY, true>(v, l.t, q % tx, q / tx, b, l.x, nxc, nyc, bc, mg_xs);
+    }
+    mg_cluster_sync();
   }
+  {  // coarsest: x = C b, a warp per row, b in shared memory (at most LMAX x 64 values)
+    const float* b = k0 == nl - 1 ? b0 : sl[nl - 1 - k0].b;
+    float* x = sl[nl - 1 - k0].x;
+    for (int j = t; j < nc; j += MGT_EX * MG_EY) mg_xs[j] = __ldcg(b + j);
+    __syncthreads();
+    const int nw = MGT_EX * MG_EY / 32, lane = t & 31;
+    for (int row = blockIdx.x * nw + (t >> 5); row < nc; row += nw * gridDim.x) {
+      float acc = 0.f;
+#pragma unroll 8
+      for (int j = lane; j < nc; j += 32) acc += __ldg(cinv + (long long)row * nc + j) * mg_xs[j];
+      acc = warp_sum(acc);
+      if (lane == 0) x[row] = acc;
+    }
+    if (nl - 1 > k0) mg_cluster_sync();
+  }
+  for (int k = nl - 2; k >= k0; --k) {
+    const MGCLev<LMAX>& l = sl[k - k0];
+    const int nxc = (l.nx + 1) / 2, nyc = (l.ny + 1) / 2, tx = (l.nx + MGT_EX - 3) / (MGT_EX - 2);
+    const MGDev v{l.nx, l.ny, L, l.gx, l.gy, l.gz, l.s, l.m, l.w};
+    const MGCLev<LMAX>& c = sl[k + 1 - k0];
+    const float *b = k == k0 ? b0 : l.b, *xc = k + 1 == nl - 1 ? c.x : c.xt;
+    float* out = k == 0 ? z : l.xt;
+    for (int q = blockIdx.x; q < mgt_tiles<MG_EY>(l.nx, l.ny); q += gridDim.x) {
+      __syncthreads();
+      float rz;
+      if (l.uni) rz = mgt_up<LMAX, true, MG_EY, true, true>(v, l.t, q % tx, q / tx, b, l.x, xc, nxc, nyc, out, mg_xs);
+      else rz = mgt_up<LMAX, false, MG_EY, true, true>(v, l.t, q % tx, q / tx, b, l.x, xc, nxc, nyc, out, mg_xs);
+      if (k == 0) part[0] += rz;
+    }
+    if (k > k0) mg_cluster_sync();
+  }
+  if (k0 != 0) return;
+  double tot[1];
+  if (!grid_reduce<float, 1>(part, partials, stride, counter, tot)) return;
+  ctl->rz_next = tot[0];
+  ctl_set_beta(ctl);
 }
 
 // coarsest level: x = C b with the dense inverse C (n x n, FP32), a warp per row
@@ -575,6 +401,7 @@ struct MGLevelH {
 struct MGHier {
   double dt = -1.0;
   std::vector<MGLevelH> lv;
+  int cluster = 0;    // blocks of k_mg_levels' cluster (0: not looked up yet)
   bool uni = false;   // finest level from the layer table
   MGUni<32> tab{};    // its coefficients and Thomas factors (first L layers used)
   // Levels whose coefficients depend only on the layer (and on which in-plane
@@ -584,6 +411,7 @@ struct MGHier {
   std::vector<char> luni;
   std::vector<MGUni<32>> ltab;
   float* cinv = nullptr;  // dense inverse of the coarsest operator
+  void* dlv = nullptr;       // levels for k_mg_levels (MGCLev<LMAX> of the stack's layer capacity)
   double* band = nullptr;  // its banded factor (rows, columns, 1/d) and the factorisation's flag
   int nc = 0;
   ~MGHier() {
@@ -593,6 +421,7 @@ struct MGHier {
     }
     if (cinv) cudaFree(cinv);
     if (band) cudaFree(band);
+    if (dlv) cudaFree(dlv);
   }
 };
 
@@ -607,6 +436,21 @@ static th_status mg_alloc(float** p, long long n) {
 }
 
 static MGDev dev_of(const MGLevelH& l, int L) { return MGDev{l.nx, l.ny, L, l.gx, l.gy, l.gz, l.s, l.m, l.w}; }
+
+// layer capacity of the kernels
+static int mg_lmax(int L) { return L <= 4 ? 4 : (L <= 6 ? 6 : (L <= 8 ? 8 : (L <= 12 ? 12 : (L <= 16 ? 16 : 32)))); }
+#define MG_LMAX(L, STMT)                                                                             \
+  switch (mg_lmax(L)) {                                                                              \
+    case 4: { constexpr int LM = 4; STMT; break; }                                                   \
+    case 6: { constexpr int LM = 6; STMT; break; }                                                   \
+    case 8: { constexpr int LM = 8; STMT; break; }                                                   \
+    case 12: { constexpr int LM = 12; STMT; break; }                                                 \
+    case 16: { constexpr int LM = 16; STMT; break; }                                                 \
+    default: { constexpr int LM = 32; STMT; break; }                                                 \
+  }
+
+template <int LMAX>
+static th_status mg_upload(thermal_grid* g, cudaStream_t s);
 
 th_status grid_ensure_mg(thermal_grid* g, double dt, cudaStream_t s) {
   TH_TRY(grid_ensure_tab(g, dt, s));
@@ -752,6 +596,7 @@ th_status grid_ensure_mg(thermal_grid* g, double dt, cudaStream_t s) {
   TH_CUDA(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
   TH_CUDA(cudaStreamSynchronize(s));
   if (hbad) return th_fail(TH_ENOCONV, "coarsest multigrid operator is not positive definite");
+  MG_LMAX(L, TH_TRY(mg_upload<LM>(g, s)));
   h->dt = key;
   g->mg_valid = true;
   return TH_OK;
@@ -778,133 +623,138 @@ static MGUni<LMAX> uni_of(const MGHier* h, int k) {
 
 static bool mg_uni(const MGHier* h, int k) { return k < (int)h->luni.size() && h->luni[k]; }
 
-// coarse layer-uniform levels of complete aggregates up to 256 x 256 columns run the
-// column-tile kernels (latency-bound sizes); the finest level and larger levels keep
-// the 4-column bandwidth kernels (measured: a 512 x 512 x 8 level is slower in
-// column tiles)
-static bool mg_ct(const thermal_grid* g, int k) {
-  const MGHier* h = g->mg;
-  return k > 0 && mg_uni(h, k) && h->lv[k].nx % 2 == 0 && h->lv[k].ny % 2 == 0 &&
-         (long long)h->lv[k].nx * h->lv[k].ny <= 65536;
-}
-
-// the vectorised kernels apply (a layer-uniform level, nx % 4 == 0, <= 12 layers:
-// 4 columns x 12 layers of the iterate and the forward sweep fit the registers)
-static bool mg_v4(const thermal_grid* g, int k) {
-  return mg_uni(g->mg, k) && g->mg->lv[k].nx % 4 == 0 && g->L <= 12;
-}
-
+// level descriptors and tables for k_mg_levels
 template <int LMAX>
-static th_status smooth(thermal_grid* g, int k, const float* b, const float* xin, const float* xc, int nxc, int nyc,
-                        float* xout, cudaStream_t s) {
-  const MGHier* h = g->mg;
-  const MGLevelH& l = h->lv[k];
-  const MGUni<LMAX> U = uni_of<LMAX>(h, k);
-  if (mg_ct(g, k)) {
-    th_launch(k_mg_smooth_ct<LMAX>, dim3((l.nx + MG_CT_X - 1) / MG_CT_X, (l.ny + MG_CT_Y - 1) / MG_CT_Y), dim3(32, LMAX), 0, s, g->ctl, l.nx, l.ny, g->L, U, b, xin, xc, nxc, nyc, xout, MG_OMEGA);
-    TH_CHECK_LAUNCH();
-    return TH_OK;
+static th_status mg_upload(thermal_grid* g, cudaStream_t s) {
+  MGHier* h = g->mg;
+  const int nl = (int)h->lv.size();
+  std::vector<MGCLev<LMAX>> d(nl);
+  std::memset((void*)d.data(), 0, sizeof(MGCLev<LMAX>) * nl);
+  for (int k = 0; k < nl; ++k) {
+    const MGLevelH& l = h->lv[k];
+    MGCLev<LMAX>& o = d[k];
+    o.nx = l.nx;
+    o.ny = l.ny;
+    o.uni = mg_uni(h, k);
+    o.gx = l.gx;
+    o.gy = l.gy;
+    o.gz = l.gz;
+    o.s = l.s;
+    o.m = l.m;
+    o.w = l.w;
+    o.x = k == 0 ? l.xt : l.x;  // the pre-smoothed iterate
+    o.xt = l.xt;
+    o.b = l.b;
+    if (o.uni) o.t = uni_of<LMAX>(h, k);
   }
-  if constexpr (LMAX == 8 || LMAX == 12) {
-    if (mg_v4(g, k)) {
-      th_launch(k_mg_smooth4<LMAX>, dim3((l.nx / 4 + 31) / 32, (l.ny + 7) / 8), dim3(32, 8), 0, s, g->ctl, l.nx, l.ny, g->L, U, b,
-                                                                                     xin, xc, nxc, nyc, xout,
-                                                                                     MG_OMEGA);
-      TH_CHECK_LAUNCH();
-      return TH_OK;
-    }
-  }
-  if (mg_uni(h, k))
-    th_launch(k_mg_smooth<LMAX, true>, col_grid(l.nx, l.ny), dim3(32, 8), 0, s, g->ctl, dev_of(l, g->L), U, b, xin, xc, nxc,
-                                                                        nyc, xout, MG_OMEGA);
-  else
-    th_launch(k_mg_smooth<LMAX, false>, col_grid(l.nx, l.ny), dim3(32, 8), 0, s, g->ctl, dev_of(l, g->L), U, b, xin, xc,
-                                                                         nxc, nyc, xout, MG_OMEGA);
-  TH_CHECK_LAUNCH();
+  auto al = [](void** p, size_t bytes) -> th_status {
+    if (*p || cudaMalloc(p, bytes) == cudaSuccess) return TH_OK;
+    cudaGetLastError();
+    *p = nullptr;
+    return th_fail(TH_ENOMEM, "multigrid level table allocation failed");
+  };
+  TH_TRY(al(&h->dlv, sizeof(MGCLev<LMAX>) * nl));
+  TH_CUDA(cudaMemcpyAsync(h->dlv, d.data(), sizeof(MGCLev<LMAX>) * nl, cudaMemcpyHostToDevice, s));
+  TH_CUDA(cudaStreamSynchronize(s));
   return TH_OK;
 }
 
+// levels k0 .. of the cycle by one cluster
 template <int LMAX>
-static th_status restrict_(thermal_grid* g, int k, const float* b, const float* x, float* bc, cudaStream_t s) {
-  const MGHier* h = g->mg;
-  const MGLevelH& l = h->lv[k];
-  const MGLevelH& c = h->lv[k + 1];
-  const MGUni<LMAX> U = uni_of<LMAX>(h, k);
-  if (mg_ct(g, k)) {
-    th_launch(k_mg_restrict_ct<LMAX>, dim3((l.nx + MG_CT_X - 1) / MG_CT_X, (l.ny + MG_CT_Y - 1) / MG_CT_Y), dim3(32, LMAX), 0, s, g->ctl, l.nx, l.ny, g->L, U, b, x, c.nx, c.ny, bc);
-    TH_CHECK_LAUNCH();
-    return TH_OK;
+static th_status mg_levels(thermal_grid* g, int k0, const float* b0, float* z, cudaStream_t s) {
+  MGHier* h = g->mg;
+  const int nl = (int)h->lv.size();
+  auto* kern = k_mg_levels<LMAX>;
+  cudaLaunchConfig_t c{};
+  c.blockDim = dim3(MGT_EX, MG_EY);
+  c.dynamicSmemBytes = mg_xs_bytes<LMAX>() + sizeof(MGCLev<LMAX>) * (nl - k0);
+  c.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  TH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.dynamicSmemBytes));
+  TH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  auto blocks = [&](int n) {
+    c.gridDim = dim3(n);
+    at.val.clusterDim.x = n;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  };
+  blocks(MG_CLUSTER);
+  if (!h->cluster) {  // once per hierarchy
+    int fits = 0;
+    if (cudaOccupancyMaxActiveClusters(&fits, kern, &c) != cudaSuccess) cudaGetLastError();
+    h->cluster = fits > 0 ? MG_CLUSTER : 8;
   }
-  if constexpr (LMAX == 8 || LMAX == 12) {
-    if (mg_v4(g, k)) {
-      th_launch(k_mg_restrict4<LMAX>, dim3((l.nx / 4 + 31) / 32, (l.ny + 7) / 8), dim3(32, 8), 0, s, g->ctl, l.nx, l.ny, g->L, U,
-                                                                                       b, x, c.nx, c.ny, bc);
-      TH_CHECK_LAUNCH();
-      return TH_OK;
-    }
-  }
-  if (mg_uni(h, k))
-    th_launch(k_mg_restrict<LMAX, true>, col_grid(l.nx, l.ny), dim3(32, 8), 0, s, g->ctl, dev_of(l, g->L), U, b, x, c.nx,
-                                                                          c.ny, bc);
-  else
-    th_launch(k_mg_restrict<LMAX, false>, col_grid(l.nx, l.ny), dim3(32, 8), 0, s, g->ctl, dev_of(l, g->L), U, b, x, c.nx,
-                                                                           c.ny, bc);
-  TH_CHECK_LAUNCH();
+  blocks(h->cluster);
+  TH_CUDA(cudaLaunchKernelEx(&c, kern, g->ctl, (const MGCLev<LMAX>*)h->dlv, g->L, k0, nl, h->nc, (const float*)h->cinv,
+                             b0, z, g->partials, g->partials_stride, g->counters));
   return TH_OK;
 }
 
-static th_status smooth_any(thermal_grid* g, int k, const float* b, const float* xin, const float* xc, int nxc,
-                            int nyc, float* xout, cudaStream_t s) {
-  if (g->L <= 8) return smooth<8>(g, k, b, xin, xc, nxc, nyc, xout, s);
-  if (g->L <= 12) return smooth<12>(g, k, b, xin, xc, nxc, nyc, xout, s);
-  if (g->L <= 16) return smooth<16>(g, k, b, xin, xc, nxc, nyc, xout, s);
-  return smooth<32>(g, k, b, xin, xc, nxc, nyc, xout, s);
+// one half of level k as a launch of its own
+template <int LMAX, bool UNI>
+static th_status mg_half(thermal_grid* g, int k, bool up, const float* b, float* x, const float* xc, float* z,
+                         cudaStream_t s) {
+  const MGHier* h = g->mg;
+  const MGLevelH &l = h->lv[k], &c = h->lv[k + 1];
+  const MGUni<LMAX> U = uni_of<LMAX>(h, k);
+  const dim3 gr((l.nx + MGT_EX - 3) / (MGT_EX - 2), (l.ny + MG_EY - 3) / (MG_EY - 2)), bl(MGT_EX, MG_EY);
+  constexpr size_t sm = mg_xs_bytes<LMAX>();
+  auto launch = [&](auto* kern, dim3 blocks, auto... a) -> th_status {
+    if (sm > (40u << 10)) TH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    th_launch(kern, blocks, bl, sm, s, a...);
+    TH_CHECK_LAUNCH();
+    return TH_OK;
+  };
+  if (!up) return launch(k_mg_down<LMAX, UNI>, gr, g->ctl, dev_of(l, g->L), U, b, x, c.nx, c.ny, c.b);
+  if (k == 0)
+    return launch(k_mg_up<LMAX, UNI, true>, std::min(gr.x * gr.y, (LMAX <= 12 ? MG_MINB : 1u) * device_sms()), g->ctl, dev_of(l, g->L), U, b, x, xc, c.nx, c.ny, z, g->partials,
+                  g->partials_stride, g->counters);
+  return launch(k_mg_up<LMAX, UNI, false>, gr, g->ctl, dev_of(l, g->L), U, b, x, xc, c.nx, c.ny, z, g->partials,
+                g->partials_stride, g->counters);
 }
 
-static th_status restrict_any(thermal_grid* g, int k, const float* b, const float* x, float* bc, cudaStream_t s) {
-  if (g->L <= 8) return restrict_<8>(g, k, b, x, bc, s);
-  if (g->L <= 12) return restrict_<12>(g, k, b, x, bc, s);
-  if (g->L <= 16) return restrict_<16>(g, k, b, x, bc, s);
-  return restrict_<32>(g, k, b, x, bc, s);
+template <int LMAX>
+static th_status mg_cycle(thermal_grid* g, const float* r, float* z, cudaStream_t s) {
+  MGHier* h = g->mg;
+  const int nl = (int)h->lv.size();
+  auto half = [&](int k, bool up) -> th_status {
+    const MGLevelH& l = h->lv[k];
+    const float* b = k == 0 ? r : l.b;
+    float* x = k == 0 ? l.xt : l.x;  // the pre-smoothed iterate
+    const float* xc = k + 1 == nl - 1 ? h->lv[k + 1].x : h->lv[k + 1].xt;
+    float* out = k == 0 ? z : l.xt;
+    return mg_uni(h, k) ? mg_half<LMAX, true>(g, k, up, b, x, xc, out, s)
+                        : mg_half<LMAX, false>(g, k, up, b, x, xc, out, s);
+  };
+  // first level of the cluster's: two tiles a block (one: 64^2 x 4 22.5 instead of 20.5 us;
+  // eight: 512^2 x 8 78 instead of 66 us)
+  int k0 = 0;
+  while (k0 < nl - 1 && mgt_tiles<MG_EY>(h->lv[k0].nx, h->lv[k0].ny) > 2 * MG_CLUSTER) ++k0;
+  for (int k = 0; k < k0; ++k) TH_TRY(half(k, false));
+  TH_TRY(mg_levels<LMAX>(g, k0, k0 == 0 ? r : h->lv[k0].b, z, s));
+  for (int k = k0 - 1; k >= 0; --k) TH_TRY(half(k, true));
+  return TH_OK;
 }
 
-// z = M^-1 r: one V-cycle (see the file comment).  Every level's pre-smoothed
-// iterate is in x (level 0: xt); the post-smoothed one goes to xt (level 0: z).
+static th_status mg_rz(thermal_grid* g, const float* r, const float* z, cudaStream_t s);
+
+// z = M^-1 r: one V-cycle (see the file comment), r^T z and beta.
 th_status mg_vcycle(thermal_grid* g, const float* r, float* z, cudaStream_t s) {
   MGHier* h = g->mg;
   if (!h || !g->mg_valid) return th_fail(TH_ESTATE, "multigrid hierarchy not built");
-  const int nl = (int)h->lv.size();
-  if (nl == 1) {
+  if (h->lv.size() == 1) {
     th_launch(k_mg_coarsest, (h->nc + 7) / 8, 256, 0, s, g->ctl, h->nc, h->cinv, r, z);
     TH_CHECK_LAUNCH();
-    return TH_OK;
+    return mg_rz(g, r, z, s);
   }
-  std::vector<const float*> B(nl);
-  std::vector<float*> X(nl);
-  B[0] = r;
-  X[0] = h->lv[0].xt;
-  for (int k = 1; k < nl; ++k) {
-    B[k] = h->lv[k].b;
-    X[k] = h->lv[k].x;
-  }
-  for (int k = 0; k + 1 < nl; ++k) {  // down: pre-smooth from zero, restrict the residual
-    const MGLevelH& l = h->lv[k];
-    const MGLevelH& c = h->lv[k + 1];
-    TH_TRY(smooth_any(g, k, B[k], nullptr, nullptr, 1, 1, X[k], s));
-    TH_TRY(restrict_any(g, k, B[k], X[k], h->lv[k + 1].b, s));
-  }
-  th_launch(k_mg_coarsest, (h->nc + 7) / 8, 256, 0, s, g->ctl, h->nc, h->cinv, B[nl - 1], X[nl - 1]);
-  TH_CHECK_LAUNCH();
-  for (int k = nl - 2; k >= 0; --k) {  // up: coarse correction (prolongated on the fly) + post-smooth
-    const MGLevelH& c = h->lv[k + 1];
-    float* out = (k == 0) ? z : h->lv[k].xt;
-    TH_TRY(smooth_any(g, k, B[k], X[k], X[k + 1], c.nx, c.ny, out, s));
-    X[k] = out;
-  }
+  MG_LMAX(g->L, return mg_cycle<LM>(g, r, z, s));
   return TH_OK;
 }
 
-th_status mg_rz(thermal_grid* g, const float* r, const float* z, cudaStream_t s) {
+// r^T z of a single-level grid's exact solve
+static th_status mg_rz(thermal_grid* g, const float* r, const float* z, cudaStream_t s) {
   const long long n = g->n;
   static int sms[64] = {0};
   int dev = 0;

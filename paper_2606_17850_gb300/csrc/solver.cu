@@ -789,8 +789,7 @@ static th_status enq_precond_tail(const Plan& P, const VecSet<TV>& V, cudaStream
   }
   if (P.pc == TH_PC_MG) {
     if constexpr (sizeof(TV) == 4) {
-      TH_TRY(mg_vcycle(g, V.r, V.zc[0], st));
-      return mg_rz(g, V.r, V.zc[0], st);
+      return mg_vcycle(g, V.r, V.zc[0], st);
     }
     return th_fail(TH_EINVAL, "the multigrid preconditioner runs in FP32");
   }

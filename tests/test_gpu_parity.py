@@ -628,6 +628,26 @@ def test_mg_vcycle_matches_oracle(nx, ny, mk, dt):
     assert np.max(np.abs(z - z_ref)) <= 2e-5 * np.max(np.abs(z_ref))
 
 
+@pytest.mark.parametrize("nx,ny,L,kmap", [(30, 6, 4, 0), (31, 7, 6, 0), (60, 13, 8, 0), (61, 12, 12, 1), (29, 5, 14, 0),
+                                          (91, 43, 20, 0), (121, 50, 5, 1), (200, 150, 8, 0), (223, 161, 6, 1)])
+def test_mg_tiles_match_oracle(nx, ny, L, kmap):
+    """The level kernels at the edges of their 30 x 6-column tiles, every layer capacity
+    (4, 6, 8, 12, 16, 32), table and per-cell coefficients, and grids with levels both in
+    launches of their own and in the cluster; FP32 against the oracle's FP64 V-cycle, with
+    the bound of test_mg_vcycle_matches_oracle."""
+    from oracle import multigrid as mg
+    st = ti.Stack(tuple(ti.si() if i % 3 == 0 else (ti.bond() if i % 3 == 1 else ti.cu(200.0)) for i in range(L)), h=1e4)
+    g = grid_of(nx, ny, st)
+    kc = _kmap(st, nx, ny, 21) if kmap else None
+    if kmap:
+        g.set_conductivity_map(cuda(kc))
+    A = disc.assemble(nx, ny, st, k_cell=kc).tocsr()
+    r = ti.random_vector(A.shape[0], 18).astype(np.float32)
+    z = g.precond(cuda(r), 0.0, precond="mg").cpu().double().numpy()
+    z_ref = mg.vcycle(mg.hierarchy(A, nx, ny, L), L, r.astype(np.float64))
+    assert np.max(np.abs(z - z_ref)) <= 2e-5 * np.max(np.abs(z_ref))
+
+
 def test_mg_vcycle_conductivity_map_matches_oracle():
     """The finest level reads per-face arrays when the grid has a per-cell map."""
     from oracle import multigrid as mg
