@@ -33,6 +33,7 @@
 #include "internal.h"
 #include "kernels_v4.cuh"
 #include "mg_device.cuh"
+#include "mg_tile.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -67,7 +68,7 @@ struct BArgs {
   int pc, k, scaled;
   int max_sweeps;    // safety cap on inner sweeps of the whole batch
   // multigrid preconditioner (pc == TH_PC_MG): every instance's hierarchy, and for
-  // each level index k the work list of 32 x 8-column tiles of the instances that
+  // each level index k the work list of 30 x 6-column tiles of the instances that
   // smooth on level k (entries [mgt_off[k], mgt_off[k+1]) of mgt: instance, tile).
   // The offsets live in device memory: an array member of this by-value argument
   // made ptxas keep the whole argument block on the stack (spill loads 292 -> 540
@@ -318,7 +319,7 @@ static __constant__ MGUni<8> c_mg_none;
 // for the tiles of instances whose inner solve is active (checked once per instance
 // run, the flag cannot change within a phase).
 template <class F>
-__device__ void mg_phase(const BArgs& A, int k, F body) {
+__device__ void mg_phase(const BArgs& A, int k, MGUni<8>& tab, F body) {
   __shared__ int s_act;
   const int tid = thread_linear_id();
   int cur = -1;
@@ -328,11 +329,17 @@ __device__ void mg_phase(const BArgs& A, int k, F body) {
     const int2 e = __ldg(A.mgt + t);
     if (e.x != cur) {
       __syncthreads();
+      __syncthreads();  // nobody is in the tile before
       if (tid == 0) s_act = active(A.inst[e.x].ctl, ACT_INNER);
-      __syncthreads();
-      act = s_act != 0;
+      const MGBLevel& l = A.mg[e.x].lv[k];
+      if (l.uni) {  // the level's table into shared memory
+        const int* src = reinterpret_cast<const int*>(&l.t);
+        for (int i = tid; i < (int)(sizeof(MGUni<8>) / 4); i += block_threads()) reinterpret_cast<int*>(&tab)[i] = __ldg(src + i);
+      }
       cur = e.x;
     }
+    __syncthreads();
+    act = s_act != 0;
     if (act) body(e.x, e.y, t);
   }
   __syncthreads();
@@ -344,44 +351,27 @@ __device__ __forceinline__ MGDev mg_dev(const MGBDesc& D, int k, int L) {
 }
 
 // z = M^-1 r for every active instance: one V-cycle (as mg_vcycle of the single-grid
-// path), instances of different depths in the same phases; the last post-smoothing
-// also reduces r^T z.  Inlined (the multigrid instantiation spills about 1.1 KB a
-// thread, yet measured faster than the cycle as an out-of-line call, 314 vs 330 ms
-// for the 64 stacks, or at two blocks per SM without the register cap, 414 ms).
+// path), instances of different depths in the same phases; the last pass also reduces
+// r^T z.  A level is two phases on shared-memory tiles (mg_tile.cuh); with a phase each
+// for smoothing and restriction, every column reading its neighbours' from global memory,
+// the 32 stacks of 128^2 x 4 to 512^2 x 8 took 147 ms, now 76 ms.
 __device__ void mg_vcycle_batched(const BArgs& A, cg::grid_group& grid) {
-  __shared__ float rowsum[8][32];
   __shared__ double red[32];
+  __shared__ MGUni<8> tab;
+  __shared__ float xs[8 * MGT_EX * TH_BY4];
   const int tid = thread_linear_id();
   for (int k = 0; k + 1 < A.mg_maxnl; ++k) {  // down: pre-smooth from zero, restrict
-    mg_phase(A, k, [&](int ii, int tile, int) {
-      const MGBDesc& D = A.mg[ii];
-      const BInst& I = A.inst[ii];
-      const MGBLevel& l = D.lv[k];
-      const int tbx = (l.nx + 31) / 32;
-      const int x = (tile % tbx) * 32 + threadIdx.x, y = (tile / tbx) * 8 + threadIdx.y;
-      const float* b = (k == 0) ? I.r : l.b;
-      float* xo = (k == 0) ? l.xt : l.x;
-      if (x < l.nx && y < l.ny) {
-        if (l.uni)
-          mg_smooth_column<8, true>(mg_dev(D, k, I.d.L), l.t, x, y, b, nullptr, nullptr, 1, 1, xo, kMGOmega, false);
-        else
-          mg_smooth_column<8, false>(mg_dev(D, k, I.d.L), c_mg_none, x, y, b, nullptr, nullptr, 1, 1, xo, kMGOmega,
-                                     false);
-      }
-    });
-    grid.sync();
-    mg_phase(A, k, [&](int ii, int tile, int) {
+    mg_phase(A, k, tab, [&](int ii, int tile, int) {
       const MGBDesc& D = A.mg[ii];
       const BInst& I = A.inst[ii];
       const MGBLevel& l = D.lv[k];
       const MGBLevel& c = D.lv[k + 1];
-      const int tbx = (l.nx + 31) / 32;
-      if (l.uni)
-        mg_restrict_tile<8, true>(mg_dev(D, k, I.d.L), l.t, tile % tbx, tile / tbx, (k == 0) ? I.r : l.b,
-                                  (k == 0) ? l.xt : l.x, c.nx, c.ny, c.b, rowsum);
-      else
-        mg_restrict_tile<8, false>(mg_dev(D, k, I.d.L), c_mg_none, tile % tbx, tile / tbx, (k == 0) ? I.r : l.b,
-                                   (k == 0) ? l.xt : l.x, c.nx, c.ny, c.b, rowsum);
+      const int tbx = (l.nx + MGT_EX - 3) / (MGT_EX - 2);
+      const float* b = (k == 0) ? I.r : l.b;
+      float* xo = (k == 0) ? l.xt : l.x;
+      const MGDev v = mg_dev(D, k, I.d.L);
+      if (l.uni) mgt_down<8, true, TH_BY4, false>(v, tab, tile % tbx, tile / tbx, b, xo, c.nx, c.ny, c.b, xs);
+      else mgt_down<8, false, TH_BY4, false>(v, c_mg_none, tile % tbx, tile / tbx, b, xo, c.nx, c.ny, c.b, xs);
     });
     grid.sync();
   }
@@ -399,26 +389,20 @@ __device__ void mg_vcycle_batched(const BArgs& A, cg::grid_group& grid) {
   }
   grid.sync();
   for (int k = A.mg_maxnl - 2; k >= 0; --k) {  // up: prolongated correction + post-smooth
-    mg_phase(A, k, [&](int ii, int tile, int t) {
+    mg_phase(A, k, tab, [&](int ii, int tile, int t) {
       const MGBDesc& D = A.mg[ii];
       const BInst& I = A.inst[ii];
       const MGBLevel& l = D.lv[k];
       const MGBLevel& c = D.lv[k + 1];
-      const int tbx = (l.nx + 31) / 32;
-      const int x = (tile % tbx) * 32 + threadIdx.x, y = (tile / tbx) * 8 + threadIdx.y;
+      const int tbx = (l.nx + MGT_EX - 3) / (MGT_EX - 2);
       const float* b = (k == 0) ? I.r : l.b;
       const float* xin = (k == 0) ? l.xt : l.x;
       const float* xc = (k + 1 == D.nl - 1) ? c.x : c.xt;
       float* out = (k == 0) ? I.zc[0] : l.xt;
-      float rz = 0.f;
-      if (x < l.nx && y < l.ny) {
-        if (l.uni)
-          rz = mg_smooth_column<8, true>(mg_dev(D, k, I.d.L), l.t, x, y, b, xin, xc, c.nx, c.ny, out, kMGOmega,
-                                         k == 0);
-        else
-          rz = mg_smooth_column<8, false>(mg_dev(D, k, I.d.L), c_mg_none, x, y, b, xin, xc, c.nx, c.ny, out,
-                                          kMGOmega, k == 0);
-      }
+      const MGDev v = mg_dev(D, k, I.d.L);
+      float rz;
+      if (l.uni) rz = mgt_up<8, true, TH_BY4, false, true>(v, tab, tile % tbx, tile / tbx, b, xin, xc, c.nx, c.ny, out, xs);
+      else rz = mgt_up<8, false, TH_BY4, false, true>(v, c_mg_none, tile % tbx, tile / tbx, b, xin, xc, c.nx, c.ny, out, xs);
       if (k == 0) {  // r^T z of the tile
         const float ws = warp_sum(rz);
         if ((tid & 31) == 0) red[tid >> 5] = (double)ws;
@@ -675,7 +659,7 @@ static th_status launch_batch(std::vector<BInst>& hi, const std::vector<thermal_
   A.k = k;
   A.scaled = opts->cheb_scaled ? 1 : 0;
   A.max_sweeps = max_sweeps;
-  // multigrid: per level index, the 32 x 8-column tiles of the instances that smooth
+  // multigrid: per level index, the 30 x 6-column tiles of the instances that smooth
   // on that level (instance by instance, so each instance's level-0 tiles are one range)
   DevArr<MGBDesc> dmg;
   DevArr<int2> dmgt, dml0;
@@ -699,7 +683,7 @@ static th_status launch_batch(std::vector<BInst>& hi, const std::vector<thermal_
       for (int i = 0; i < n; ++i) {
         const MGBDesc& D = (*mgd)[i];
         if (lvl > D.nl - 2) continue;
-        const int nt = ((D.lv[lvl].nx + 31) / 32) * ((D.lv[lvl].ny + 7) / 8);
+        const int nt = mgt_tiles<TH_BY4>(D.lv[lvl].nx, D.lv[lvl].ny);
         if (lvl == 0) l0[i] = make_int2((int)lst.size(), nt);
         for (int t = 0; t < nt; ++t) lst.push_back(make_int2(i, t));
       }

@@ -7,10 +7,11 @@
 // instead of five, and the two passes of a level's way down (smoothing from zero, residual
 // and restriction) need b only once: the ring's columns are smoothed again, which is local
 // to a column.  Both halves work on any nx, ny (aggregates at an odd edge are incomplete)
-// and on either coefficient source (MGC).  CG: the vectors were written by other blocks of
+// and on either coefficient source.  CG: the vectors were written by other blocks of
 // the running kernel (loads that bypass L1).
 //
-// The arithmetic and its order are those of mg_smooth_column and mg_restrict_tile.
+// Order of a cell's product: s x, then the x, y and z faces (+ before -); an aggregate is
+// summed x pairs first.
 #pragma once
 
 #include "mg_device.cuh"
@@ -22,8 +23,7 @@ __device__ __forceinline__ float mgt_ld(const float* p) {
   return CG ? __ldcg(p) : *p;
 }
 
-// columns and rows of results in one tile, tiles of a level
-template <int EY> __host__ __device__ constexpr int mgt_rows() { return EY - 2; }
+// tiles of a level
 template <int EY>
 __host__ __device__ __forceinline__ int mgt_tiles(int nx, int ny) {
   return ((nx + MGT_EX - 3) / (MGT_EX - 2)) * ((ny + EY - 3) / (EY - 2));
