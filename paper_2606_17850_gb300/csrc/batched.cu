@@ -443,9 +443,10 @@ __device__ void mg_vcycle_batched(const BArgs& A, cg::grid_group& grid) {
 // phases need the occupancy more than the rarely run FP64 residual phase needs
 // registers (measured: 0.92 s vs 1.12 s with two blocks per SM for the 64 stacks).
 // MGP: the multigrid instantiation (its V-cycle phases are compiled only there, so
-// the other preconditioners keep their register allocation)
+// the other preconditioners keep their register allocation); four blocks per SM there (its
+// tile passes wait on latency: 32 stacks 91.6 / 76.2 / 74.3 ms at 2 / 3 / 4 blocks)
 template <typename TP, bool MGP>
-__global__ void __launch_bounds__(TH_BX* TH_BY4, 3) k_batched(BArgs A) {
+__global__ void __launch_bounds__(TH_BX* TH_BY4, MGP ? 4 : 3) k_batched(BArgs A) {
   cg::grid_group grid = cg::this_grid();
   const int rz_here = (A.pc == TH_PC_NONE || A.pc == TH_PC_JACOBI || (A.pc == TH_PC_CHEB && A.k == 1)) ? 1 : 0;
   auto zfinal = [&](const BInst& I) -> const float* {
