@@ -468,8 +468,9 @@ th_status grid_ensure_workspace(thermal_grid* g, bool need64, cudaStream_t s) {
     TH_TRY(dalloc(&g->thn_hi, n));
     TH_TRY(dalloc(&g->thn_lo, n));
     const dim3 gb = grid_blocks(g);
-    // one slot per block of any reducing kernel: cell blocks, or resident blocks
-    g->partials_stride = std::max((int)(gb.x * gb.y * gb.z), 8 * device_sms());
+    // one slot per block of any reducing kernel: cell blocks, or resident blocks (the
+    // streaming chunks' one-warp blocks: at most 14 per SM, and a strip each at least)
+    g->partials_stride = std::max((int)(gb.x * gb.y * gb.z), 16 * device_sms());
     TH_TRY(dalloc(&g->partials, (size_t)4 * g->partials_stride + 64));
     TH_TRY(dalloc(&g->counters, 64));
     TH_CUDA(cudaMemsetAsync(g->counters, 0, 64 * sizeof(unsigned), s));

@@ -214,6 +214,27 @@ void graph_cache_free(GraphCache* c);
 th_status solver_cheb_coeffs(thermal_grid* g, double dt, const thermal_solve_opts* o, std::vector<float>& c1,
                              std::vector<float>& c2, float* inv_theta, double* lmin, double* lmax, cudaStream_t s);
 int device_sms();
+// 3-D tensor map of one FP32 field (x fastest, then y, then layer) with a box of bw x bh
+// columns x L layers; cells outside the grid read as zero.  TH_EINVAL unless nx % 4 == 0
+// and the base is 16-byte aligned.
+struct CUtensorMap_st;
+th_status tensor_map_3d(struct CUtensorMap_st* m, const Dims& d, const float* base, int bw, int bh);
+// One launch of fused Chebyshev steps (kernels_stream.cuh): coefficients of its steps,
+// vectors, and whether it starts the polynomial / ends it (r^T z, no z_{m-1} output).
+struct StreamChunk {
+  int steps;
+  bool first, last;
+  float c1[4], c2[4], z1s;
+  int expire_test;
+  const float *in_cur, *in_prev, *r;
+  float *out_cur, *out_prev;
+};
+struct StreamCut { int strips, rows, warps; };
+StreamCut cheb_stream_cut(int nx, int ny, int L);
+bool cheb_stream_pays(int nx, int ny, int L);  // rather than k_cheb_tb's tiles
+th_status cheb_stream_4(thermal_grid* g, const Dims& d, const StreamChunk& c, cudaStream_t s);
+th_status cheb_stream_6(thermal_grid* g, const Dims& d, const StreamChunk& c, cudaStream_t s);
+th_status cheb_stream_8(thermal_grid* g, const Dims& d, const StreamChunk& c, cudaStream_t s);
 // pcg_oc.cu: the whole FP32 inner PCG with the Chebyshev preconditioner (solve = 1: on
 // r, the correction in d32), or one application of it (solve = 0: z = M^-1 r), as one
 // cooperative launch over tiles that stay on chip; layer-uniform grids whose tiles fit

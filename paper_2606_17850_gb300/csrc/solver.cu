@@ -54,6 +54,7 @@ struct Plan {
   // pool of four FP32 buffers {zc0, zc1, zc2, mu} (indices 0..3)
   struct Chunk { int steps, m0, in_cur, in_prev, out_cur, out_prev; };
   bool fused = false;  // temporal blocking active
+  bool stream = false;  // the chunks run as register streams (kernels_stream.cuh), not tiles
   bool oc = false;     // inner PCG on chip (pcg_oc.cu)
   OCShape oc_tile{0, 0};
   int tb_lmax = 8;  // layer capacity of the fused kernel (8: 32 x 32 tiles, 12: 32 x 24)
@@ -398,6 +399,7 @@ static th_status make_plan(thermal_grid* g, double dt, const thermal_solve_opts*
       P.tb_lmax = g->L <= 8 ? 8 : ((g->L <= 12 && P.uni) ? 12 : 0);
       if (P.tb_lmax > 0) {
         P.fused = true;
+        P.stream = P.uni && cheb_stream_pays(g->nx, g->ny, g->L);
         int cur = 0, prev = -1, m = 1, left = P.k - 1;
         while (left > 0) {
           const int st = std::min(fuse, left);
@@ -533,22 +535,24 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensormap_encoder() {
   return fn;
 }
 
-// 3-D map of one FP32 field (x fastest, then y, then layer) with a box of
-// TB_BW x ey x L cells; cells outside the grid read as zero.
-static th_status tb_map(CUtensorMap* m, const Dims& d, const float* base, int ey) {
+th_status tensor_map_3d(CUtensorMap* m, const Dims& d, const float* base, int bw, int bh) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensormap_encoder();
   if (!enc) return th_fail(TH_ECUDA, "cuTensorMapEncodeTiled is not available");
   if (((uintptr_t)base & 15) != 0 || (d.nx % 4) != 0)
     return th_fail(TH_EINVAL, "tensor map needs a 16-byte aligned base and nx %% 4 == 0");
   const cuuint64_t dims[3] = {(cuuint64_t)d.nx, (cuuint64_t)d.ny, (cuuint64_t)d.L};
   const cuuint64_t strides[2] = {(cuuint64_t)d.nx * sizeof(float), (cuuint64_t)d.pxy * sizeof(float)};
-  const cuuint32_t box[3] = {(cuuint32_t)TB_BW, (cuuint32_t)ey, (cuuint32_t)d.L};
+  const cuuint32_t box[3] = {(cuuint32_t)bw, (cuuint32_t)bh, (cuuint32_t)d.L};
   const cuuint32_t es[3] = {1, 1, 1};
   const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void*)base, dims, strides, box, es,
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return th_fail(TH_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
   return TH_OK;
+}
+
+static th_status tb_map(CUtensorMap* m, const Dims& d, const float* base, int ey) {
+  return tensor_map_3d(m, d, base, TB_BW, ey);
 }
 
 static int sm_count() {
@@ -699,6 +703,28 @@ static th_status tb_chunk(const Plan& P, const VecSet<float>& V, cudaStream_t st
   return last ? tb_steps<LM, EY, true, true, false>(P, V, st, c) : tb_steps<LM, EY, true, false, false>(P, V, st, c);
 }
 
+static th_status stream_chunk(const Plan& P, const VecSet<float>& V, cudaStream_t st, const Plan::Chunk& c, bool last) {
+  float* pool[4] = {V.zc[0], V.zc[1], V.zc[2], V.mu};
+  StreamChunk q{};
+  q.steps = c.steps;
+  q.first = tb_first(c);
+  q.last = last;
+  for (int j = 0; j < c.steps; ++j) {
+    q.c1[j] = (float)P.c1[c.m0 + j];
+    q.c2[j] = (float)P.c2[c.m0 + j];
+  }
+  q.z1s = (float)P.inv_theta;
+  q.expire_test = P.expire_test;
+  q.in_cur = pool[c.in_cur];
+  q.in_prev = c.in_prev >= 0 ? pool[c.in_prev] : pool[c.in_cur];
+  q.r = V.r;
+  q.out_cur = pool[c.out_cur];
+  q.out_prev = c.out_prev >= 0 ? pool[c.out_prev] : nullptr;
+  if (P.d.L <= 4) return cheb_stream_4(P.g, P.d, q, st);
+  if (P.d.L <= 6) return cheb_stream_6(P.g, P.d, q, st);
+  return cheb_stream_8(P.g, P.d, q, st);
+}
+
 // the whole inner solve (solve = 1) or one application of the polynomial, on chip
 static th_status oc_enqueue(const Plan& P, cudaStream_t st, int solve, const float* r, float* z) {
   const OCRun o{P.oc_tile, solve, P.k, r, z, P.c1.data(), P.c2.data(), P.inv_theta, P.expire_test};
@@ -709,7 +735,8 @@ static th_status tb_chain(const Plan& P, const VecSet<float>& V, cudaStream_t st
   for (size_t ci = 0; ci < P.chunks.size(); ++ci) {
     const bool last = (ci + 1 == P.chunks.size());
     const Plan::Chunk& c = P.chunks[ci];
-    if (!P.uni) TH_TRY(tbf_chunk(P, V, st, c, last));
+    if (P.stream) TH_TRY(stream_chunk(P, V, st, c, last));
+    else if (!P.uni) TH_TRY(tbf_chunk(P, V, st, c, last));
     else if (P.tb_lmax == 8) TH_TRY((tb_chunk<8, 32>(P, V, st, c, last)));
     else TH_TRY((tb_chunk<12, 24>(P, V, st, c, last)));
   }
@@ -1717,6 +1744,7 @@ extern "C" th_status thermal_kernel_time(thermal_grid* g, int kernel, int reps, 
     if (kernel >= 13) {
       // one inner chunk: z_m, z_{m-1}, r in; z_{m+S}, z_{m+S-1} out (no reduction)
       const Plan::Chunk c{kernel == 13 ? 4 : (kernel == 14 ? 2 : 3), 1, 0, 1, 2, 3};
+      if (P.stream) return stream_chunk(P, V, s, c, false);
       if (P.tb_lmax == 8) return tb_chunk<8, 32>(P, V, s, c, false);
       return tb_chunk<12, 24>(P, V, s, c, false);
     }

@@ -317,6 +317,21 @@ def test_fused_chebyshev_equals_stepwise(k, dt, mk):
         assert (zf - z1).abs().max().item() <= tol * scale, fuse
 
 
+@pytest.mark.parametrize("nx,ny,mk", [(772, 771, "c2"), (1024, 1024, "c2"), (2052, 263, "c2"), (260, 2051, "l7"),
+                                      (448, 451, "c1"), (1028, 520, "l6"), (1084, 700, "l5")])
+def test_streaming_chebyshev_equals_stepwise(nx, ny, mk):
+    """Grids large enough for the streaming chunks: every chunk length as first, inner and
+    last one, strips that end inside and at the grid's edge, uneven row cuts, 4 to 8
+    layers; against one launch per step with the bound of the fused chunks."""
+    st = STACKS[mk]()
+    g = grid_of(nx, ny, st)
+    r = cuda(ti.random_vector(nx * ny * st.L, 5).astype(np.float32))
+    for k, fuse, dt in ((2, 0, 0.0), (4, 0, 1e-4), (5, 4, 0.0), (12, 0, 1e-4), (12, 2, 0.0), (12, 3, 1e-4), (16, 0, 0.0)):
+        z1 = g.precond(r, dt, precond="cheb", cheb_degree=k, cheb_fuse=1)
+        zf = g.precond(r, dt, precond="cheb", cheb_degree=k, cheb_fuse=fuse)
+        assert (zf - z1).abs().max().item() <= max(1e-6, 2.5e-7 * k) * z1.abs().max().item(), (k, fuse, dt)
+
+
 @pytest.mark.parametrize("k", [2, 5, 8, 12])
 @pytest.mark.parametrize("dt", [0.0, 1e-4])
 @pytest.mark.parametrize("mk", ["c2", "c1", "l5", "l7"])
