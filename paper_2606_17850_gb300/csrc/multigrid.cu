@@ -505,10 +505,6 @@ th_status grid_ensure_mg(thermal_grid* g, double dt, cudaStream_t s) {
                                             c.own_gz, c.s);
     TH_CHECK_LAUNCH();
   }
-  for (auto& l : h->lv) {
-    k_mg_zfactors<<<col_grid(l.nx, l.ny), dim3(32, 8), 0, s>>>(l.nx, l.ny, L, l.gx, l.gy, l.gz, l.s, l.m, l.w);
-    TH_CHECK_LAUNCH();
-  }
   // layer-uniform levels: coefficients and Thomas factors per in-plane case
   h->uni = g->uniform;
   const size_t nlv = h->lv.size();
@@ -569,6 +565,12 @@ th_status grid_ensure_mg(thermal_grid* g, double dt, cudaStream_t s) {
       h->luni[k + 1] = 1;
     }
     h->tab = h->ltab[0];
+  }
+  for (size_t k = 0; k < nlv; ++k) {  // a layer-uniform level's factors are in its table
+    const MGLevelH& l = h->lv[k];
+    if (h->luni[k]) continue;
+    k_mg_zfactors<<<col_grid(l.nx, l.ny), dim3(32, 8), 0, s>>>(l.nx, l.ny, L, l.gx, l.gy, l.gz, l.s, l.m, l.w);
+    TH_CHECK_LAUNCH();
   }
   // dense inverse of the coarsest operator (at most MG_COARSEST^2 columns x L layers)
   const MGLevelH& c = h->lv.back();
