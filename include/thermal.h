@@ -103,14 +103,15 @@ typedef struct thermal_solve_opts {
                        /* 4 T_{n-2} - T_{n-3} (2, 3: mixed path with nx % 4 == 0, linear       */
                        /* elsewhere); the order is lowered while the history is short and to */
                        /* the steps taken since the power map last switched (0)               */
-  int cheb_fuse;       /* Chebyshev steps per launch (temporal blocking in shared memory) on  */
-                       /* grids with nx % 4 == 0: layer table up to 12 layers, per-face arrays */
-                       /* up to 8 (not with the BF16 coefficients): 0 auto (4), 1 one step   */
+  int cheb_fuse;       /* Chebyshev steps per launch (temporal blocking) on grids with       */
+                       /* nx % 4 == 0: layer table up to 12 layers, per-face arrays up to 8   */
+                       /* (not with the BF16 coefficients): 0 auto (small layer-table grids,  */
+                       /* any nx: the whole inner solve in one launch; else 4), 1 one step    */
                        /* per launch, 2..4 (0)                                                */
   int ad_check;        /* ADAPTIVE: PCG iterations between true-residual evaluations of the   */
                        /* switching criterion, rounded up to even; 0: 20 steady, 6 transient  */
                        /* (the paper's 20 and 5 on the two-iteration loop body) (0)           */
-  int test_wait_expire; /* test hook, 0 in normal use: 1 makes every CTA of the fused        */
+  int test_wait_expire; /* test hook, 0 in normal use: 1 makes every CTA of a fused          */
                        /* Chebyshev kernel first wait on a barrier phase that nothing        */
                        /* completes, so its bounded wait runs out after 2 ms and the solve   */
                        /* ends with TH_ECUDA ("device wait timed out"); the grid stays usable */
