@@ -27,9 +27,8 @@ bool cheb_stream_pays(int nx, int ny, int L) {
   if (L > 8 || nx % 4 != 0 || (long long)nx * ny >= (1LL << 30)) return false;
   const StreamCut c = cheb_stream_cut(nx, ny, L);
   const int sms = device_sms(), n = (c.warps + 4 * sms - 1) / (4 * sms);
-  const int i = L <= 4 ? 0 : (L <= 6 ? 1 : 2);
-  const double row = (const double[]){0.5, 0.75, 0.75}[i] + (const double[]){0.25, 0.38, 0.4}[i] * n;
-  const double round = (const double[]){3.8, 4.05, 4.2}[i];
+  const double row = L <= 4 ? 0.5 + 0.25 * n : (L <= 6 ? 0.75 + 0.38 * n : 0.75 + 0.4 * n);
+  const double round = L <= 4 ? 3.8 : (L <= 6 ? 4.05 : 4.2);
   const long long tiles = (long long)((nx + 23) / 24) * ((ny + 23) / 24);
   return (c.rows + 2 * TB_H) * row < 2.0 + round * (double)((tiles + sms - 1) / sms);
 }

@@ -1692,10 +1692,13 @@ extern "C" th_status thermal_kernel_time(thermal_grid* g, int kernel, int reps, 
   thermal_default_opts(&o);
   o.precond = ((kernel >= 13 && kernel <= 15) || kernel >= 20) ? TH_PC_CHEB : (kernel == 19 ? TH_PC_MG : TH_PC_JACOBI);
   o.cheb_degree = 5;  // one chunk of four fused steps
+  o.cheb_fuse = TB_H;  // the chunk kernels, on a grid that solves on chip too
   o.precision = (kernel >= 5 && kernel <= 7) ? TH_PREC_FP64
                 : ((kernel >= 16 && kernel <= 18) ? TH_PREC_ADAPTIVE : TH_PREC_MIXED_IR);
   Plan P;
   TH_TRY(make_plan(g, dt, &o, TH_F32, dt > 0.0, P, s));
+  if (kernel >= 13 && kernel <= 15 && !P.fused)
+    return th_fail(TH_EINVAL, "fused Chebyshev steps hold at most 12 layers");
   TH_TRY(ensure_stage(g, sizeof(float) * (size_t)g->n));
   TH_TRY(grid_ensure_workspace(g, true, s));
   const long long n = g->n;

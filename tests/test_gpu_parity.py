@@ -1158,3 +1158,19 @@ def test_onchip_wait_expiry_and_limits(graph):
     with pytest.raises(ThermalError) as e:
         g.solve_steady(P, tol_rel=1e-10, max_outer=2, max_inner=3, **o)
     assert e.value.status == 4
+
+
+@pytest.mark.parametrize("nx,ny,L", [(64, 40, 4), (76, 36, 10), (132, 20, 12), (36, 20, 14)])
+def test_chunk_timing_on_small_grids(nx, ny, L):
+    """The chunk kernels' timing on grids that solve on chip: the tile form of the stack's
+    layer capacity runs; a stack of more than 12 layers has none."""
+    from paper_2606_17850_gb300 import ThermalError
+    st = ti.Stack(tuple(ti.si() if i % 2 == 0 else ti.bond() for i in range(L)), h=1e4)
+    g = grid_of(nx, ny, st)
+    for name in ("cheb_tb4", "cheb_tb3", "cheb_tb2"):
+        if L <= 12:
+            assert g.kernel_time(name, reps=2, dt=1e-4) > 0
+        else:
+            with pytest.raises(ThermalError) as e:
+                g.kernel_time(name, reps=2, dt=1e-4)
+            assert e.value.status == 1
