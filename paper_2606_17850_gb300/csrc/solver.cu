@@ -328,8 +328,9 @@ th_status solver_cheb_coeffs(thermal_grid* g, double dt, const thermal_solve_opt
 
 // ------------------------------------------------------------------ plan setup
 
+// apply_only: the plan of one preconditioner application (nothing else of it is launched)
 static th_status make_plan(thermal_grid* g, double dt, const thermal_solve_opts* o, int pdtype, bool transient,
-                           Plan& P, cudaStream_t s) {
+                           Plan& P, cudaStream_t s, bool apply_only = false) {
   P.g = g;
   P.d = grid_dims(g);
   P.gb = grid_blocks(g);
@@ -359,7 +360,15 @@ static th_status make_plan(thermal_grid* g, double dt, const thermal_solve_opts*
   if (P.prec == TH_PREC_FP64) TH_TRY(grid_ensure_dg64(g, dt, s));
   P.v4 = (g->nx % 4 == 0);
   P.uni = g->uniform;
-  if (P.v4) {
+  // a grid whose tiles fit the SMs keeps the inner PCG on chip (any nx); an explicit
+  // cheb_fuse asks for the tile kernels
+  if (P.pc == TH_PC_CHEB && P.prec != TH_PREC_FP64 && !P.ad && P.scaled && P.uni && o->cheb_fuse == 0) {
+    P.oc_tile = oc_shape(g->nx, g->ny, g->L, P.k);
+    P.oc = P.oc_tile.rows > 0;
+  }
+  // one application on chip needs none of the z-walk kernels (their chunk is tuned once per
+  // grid, by timing: most of a first call on a small grid)
+  if (P.v4 && !(apply_only && P.oc)) {
     TH_TRY(tune_zchunk(g, s));
     P.zc = g->zc_tuned;
     P.tb4 = dim3(TH_BX, TH_BY4);
@@ -379,12 +388,6 @@ static th_status make_plan(thermal_grid* g, double dt, const thermal_solve_opts*
     cheb_coeffs(P.lmin, P.lmax, P.k, P.c1, P.c2, &P.inv_theta);
     P.pc_spmv = P.k - 1;
     const int fuse = o->cheb_fuse == 0 ? TB_H : o->cheb_fuse;
-    // a grid whose tiles fit the SMs keeps the inner PCG on chip (any nx); an explicit
-    // cheb_fuse asks for the tile kernels
-    if (P.prec != TH_PREC_FP64 && !P.ad && P.scaled && P.uni && o->cheb_fuse == 0) {
-      P.oc_tile = oc_shape(g->nx, g->ny, g->L, P.k);
-      P.oc = P.oc_tile.rows > 0;
-    }
     // fused chunks exist for the Jacobi-scaled form (the default); the unscaled
     // polynomial of the paper runs one step per launch
     // (per-face grids: FP32 faces, so not the BF16-coefficient precision)
@@ -1657,8 +1660,9 @@ extern "C" th_status thermal_precond_apply(thermal_grid* g, double dt, const the
   thermal_solve_opts o = *opts;
   o.precision = (opts->precision == TH_PREC_MIXED_IR_BF16) ? TH_PREC_MIXED_IR_BF16 : TH_PREC_MIXED_IR;
   Plan P;
-  TH_TRY(make_plan(g, dt, &o, TH_F32, dt > 0.0, P, s));
-  if (P.oc && (z + g->n <= r || r + g->n <= z)) {  // one launch from r to z
+  const bool apart = z + g->n <= r || r + g->n <= z;
+  TH_TRY(make_plan(g, dt, &o, TH_F32, dt > 0.0, P, s, apart));
+  if (P.oc && apart) {  // one launch from r to z
     TH_TRY(oc_enqueue(P, s, 0, r, z));
     TH_CUDA(cudaStreamSynchronize(s));
     return TH_OK;
