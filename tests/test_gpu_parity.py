@@ -1174,3 +1174,34 @@ def test_chunk_timing_on_small_grids(nx, ny, L):
             with pytest.raises(ThermalError) as e:
                 g.kernel_time(name, reps=2, dt=1e-4)
             assert e.value.status == 1
+
+
+@pytest.mark.parametrize("nx,ny,pc,k,kmap", [(64, 40, "cheb", 9, 0), (64, 40, "mg", 1, 0), (37, 21, "cheb", 9, 0),
+                                             (76, 37, "cheb", 6, 1), (772, 768, "cheb", 9, 0), (8, 5, "mg", 1, 0)])
+def test_precond_buffers(nx, ny, pc, k, kmap):
+    """The application reads r and writes z in the caller's buffers where it can: the same
+    vector through buffers at any 4-byte offset and in place (z = r), r untouched."""
+    import ctypes as C
+    from paper_2606_17850_gb300 import _lib, api
+    st = ti.stack_c2()
+    g = grid_of(nx, ny, st)
+    if kmap:
+        g.set_conductivity_map(cuda(_kmap(st, nx, ny, 21)))
+    o = dict(precond=pc, cheb_degree=k)
+    r0 = cuda(ti.random_vector(g.n, 31).astype(np.float32))
+    z0 = g.precond(r0, 1e-4, **o)
+    opts, lib = api.make_opts(**o), _lib.load()
+    for ro, zo in ((0, 0), (1, 0), (0, 3), (2, 1)):
+        buf = torch.zeros(2, g.n + 8, device="cuda")
+        r, z = buf[0, ro:ro + g.n], buf[1, zo:zo + g.n]
+        r.copy_(r0)
+        assert lib.thermal_precond_apply(g.handle, 1e-4, C.byref(opts), C.c_void_p(r.data_ptr()),
+                                         C.c_void_p(z.data_ptr()), None) == 0
+        torch.cuda.synchronize()
+        assert torch.equal(z, z0) and torch.equal(r, r0), (ro, zo)
+        assert buf[1, :zo].abs().sum() == 0 and buf[1, zo + g.n:].abs().sum() == 0
+    r = r0.clone()
+    assert lib.thermal_precond_apply(g.handle, 1e-4, C.byref(opts), C.c_void_p(r.data_ptr()),
+                                     C.c_void_p(r.data_ptr()), None) == 0
+    torch.cuda.synchronize()
+    assert torch.equal(r, z0)
