@@ -11,6 +11,8 @@
 #include <cstring>
 #include <new>
 
+#include <cudaTypedefs.h>
+
 #include "internal.h"
 #include "dfloat.cuh"
 #include "kernels_ad.cuh"
@@ -102,6 +104,43 @@ bool is_device_pointer(const void* p) {
     return false;
   }
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+}
+
+// Managed memory counts as memory of the device that asks.
+BufRange buffer_range(const void* p, int device) {
+  BufRange b{(uintptr_t)p, -1, 0, 0};
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return b;
+  }
+  if (a.type != cudaMemoryTypeDevice && a.type != cudaMemoryTypeManaged) return b;
+  static const PFN_cuMemGetAddressRange_v3020 range = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 3020, cudaEnableDefault, &q) != cudaSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return (PFN_cuMemGetAddressRange_v3020)f;
+  }();
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  if (!range || range(&base, &size, (CUdeviceptr)p) != CUDA_SUCCESS) return b;
+  b.device = a.type == cudaMemoryTypeManaged ? device : a.device;
+  b.base = (uintptr_t)base;
+  b.size = size;
+  return b;
+}
+
+// A copy takes buffers of another device, at any byte, and refuses those that end before
+// their `bytes`; a kernel would fault on them.
+extern "C" int th_direct_buffers(const BufRange* r, const BufRange* z, size_t bytes, int device) {
+  for (const BufRange* b : {r, z})
+    if (b->device != device || b->p < b->base || bytes > b->size || b->p - b->base > b->size - bytes) return 0;
+  if (r->p < z->p + bytes && z->p < r->p + bytes) return 0;  // overlap
+  const uintptr_t low = r->p | z->p;
+  return (low & 3u) ? 0 : ((low & 15u) ? 1 : 2);
 }
 
 // ------------------------------------------------------------------ kernels

@@ -198,6 +198,18 @@ th_status mg_batch_levels(thermal_grid* g, MGBDesc* out, cudaStream_t s);
 dim3 grid_blocks(const thermal_grid* g);
 Dims grid_dims(const thermal_grid* g);
 bool is_device_pointer(const void* p);
+// A caller's buffer as the driver knows it: the device whose memory it is (-1: not device
+// memory) and the allocation around it.
+struct BufRange {
+  uintptr_t p;
+  int device;
+  uintptr_t base;
+  size_t size;
+};
+BufRange buffer_range(const void* p, int device);
+// Whether kernels on `device` may read r and write z where they are: 0 no (copies check
+// and convert whatever the caller has), 1 by 4-byte words, 2 by 16-byte words as well.
+extern "C" int th_direct_buffers(const BufRange* r, const BufRange* z, size_t bytes, int device);
 th_status validate_opts(const thermal_solve_opts* o);
 
 // solver.cu

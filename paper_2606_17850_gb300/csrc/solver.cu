@@ -1660,9 +1660,10 @@ extern "C" th_status thermal_precond_apply(thermal_grid* g, double dt, const the
   thermal_solve_opts o = *opts;
   o.precision = (opts->precision == TH_PREC_MIXED_IR_BF16) ? TH_PREC_MIXED_IR_BF16 : TH_PREC_MIXED_IR;
   Plan P;
-  // read r and write z in place of copies: buffers that do not overlap, in device memory
-  const bool direct = (z + g->n <= r || r + g->n <= z) && is_device_pointer(r) && is_device_pointer(z);
-  TH_TRY(make_plan(g, dt, &o, TH_F32, dt > 0.0, P, s, direct));
+  // read r and write z in place of copies, where kernels of this grid's device can
+  const BufRange br = buffer_range(r, g->device), bz = buffer_range(z, g->device);
+  const int direct = th_direct_buffers(&br, &bz, sizeof(float) * (size_t)g->n, g->device);
+  TH_TRY(make_plan(g, dt, &o, TH_F32, dt > 0.0, P, s, direct > 0));
   if (P.oc && direct) {  // one launch from r to z
     TH_TRY(oc_enqueue(P, s, 0, r, z));
     TH_CUDA(cudaStreamSynchronize(s));
@@ -1677,7 +1678,7 @@ extern "C" th_status thermal_precond_apply(thermal_grid* g, double dt, const the
   // want), without the start of an inner solve and the two copies.  Chebyshev-29 on
   // 1024 x 1024 x 8: 365 -> 318 us, a V-cycle on 640 x 384 x 8 130 -> 102 us, Chebyshev-16
   // on a 500 x 333 x 6 conductivity map 162 -> 127 us.
-  if (direct && (((uintptr_t)r | (uintptr_t)z) & 15u) == 0 && (P.fused || P.pc == TH_PC_MG)) {
+  if (direct == 2 && (P.fused || P.pc == TH_PC_MG)) {
     V.r = const_cast<float*>(r);
     if (P.pc == TH_PC_CHEB && P.zfin == 3) V.mu = z;
     else V.zc[P.pc == TH_PC_CHEB ? P.zfin : 0] = z;

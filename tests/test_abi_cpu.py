@@ -151,3 +151,34 @@ def test_noalloc_rejects_before_any_device_work(lib):
     for y in (a, C.c_void_p((1 << 20) + 32)):
         assert f(4, 4, 1, a, a, a, s_arr, a, y, xAx, None) == _lib.TH_EINVAL
         assert b"overlap" in lib.thermal_last_error()
+
+
+def test_precond_buffers_read_in_place_only_where_kernels_can(lib):
+    """A preconditioner application hands the caller's buffers to its kernels only when both
+    are whole inside allocations of the grid's device, apart, and on 4-byte words (1) or
+    16-byte words (2); everything else goes through copies (0), which check and convert."""
+    class Buf(C.Structure):
+        _fields_ = [("p", C.c_void_p), ("device", C.c_int), ("base", C.c_void_p), ("size", C.c_size_t)]
+
+    n = 4096
+    f = lib.th_direct_buffers
+    f.restype, f.argtypes = C.c_int, [C.POINTER(Buf), C.POINTER(Buf), C.c_size_t, C.c_int]
+
+    def ask(r=(0, 0, n), z=(0, 0, n), device=0, rb=1 << 20, zb=1 << 30):
+        (ro, rd, rs), (zo, zd, zs) = r, z   # offset in the allocation, device, its size
+        return f(Buf(rb + ro, rd, rb, rs), Buf(zb + zo, zd, zb, zs), n, device)
+
+    assert ask() == 2 and ask(r=(16, 0, n + 16)) == 2 and ask(device=3, r=(0, 3, n), z=(0, 3, n)) == 2
+    assert ask(r=(4, 0, n + 4)) == 1 and ask(z=(8, 0, n + 8)) == 1
+    for o in (1, 2, 3, 6):                                       # not on a word
+        assert ask(r=(o, 0, 2 * n)) == 0 and ask(z=(o, 0, 2 * n)) == 0
+    assert ask(r=(0, 1, n)) == 0 and ask(z=(0, 1, n)) == 0       # another device's memory
+    assert ask(device=1) == 0
+    assert ask(r=(0, -1, 0)) == 0 and ask(z=(0, -1, 0)) == 0     # not device memory
+    assert ask(r=(0, 0, n - 4)) == 0 and ask(z=(16, 0, n)) == 0  # ends before its n bytes
+    assert ask(r=(n, 0, n)) == 0 and ask(r=(2 * n, 0, n)) == 0
+    same = dict(rb=1 << 20, zb=1 << 20)
+    assert ask(r=(0, 0, 4 * n), z=(0, 0, 4 * n), **same) == 0    # in place, and overlapping
+    assert ask(r=(0, 0, 4 * n), z=(n - 16, 0, 4 * n), **same) == 0
+    assert ask(r=(n - 4, 0, 4 * n), z=(0, 0, 4 * n), **same) == 0
+    assert ask(r=(0, 0, 4 * n), z=(n, 0, 4 * n), **same) == 2

@@ -1205,3 +1205,24 @@ def test_precond_buffers(nx, ny, pc, k, kmap):
                                      C.c_void_p(r.data_ptr()), None) == 0
     torch.cuda.synchronize()
     assert torch.equal(r, z0)
+
+
+@pytest.mark.parametrize("nx,ny,pc,k", [(64, 40, "cheb", 9), (37, 21, "cheb", 9), (64, 40, "mg", 1)])
+def test_precond_buffers_at_any_byte(nx, ny, pc, k):
+    """Buffers that are not on a 4-byte word go through copies: the same vector."""
+    import ctypes as C
+    from paper_2606_17850_gb300 import _lib, api
+    g = grid_of(nx, ny, ti.stack_c2())
+    o = dict(precond=pc, cheb_degree=k)
+    r0 = cuda(ti.random_vector(g.n, 31).astype(np.float32))
+    z0 = g.precond(r0, 1e-4, **o)
+    opts, lib = api.make_opts(**o), _lib.load()
+    raw = r0.view(torch.uint8)
+    for ro, zo in ((2, 0), (0, 1), (3, 2)):
+        buf = torch.zeros(2, 4 * g.n + 64, dtype=torch.uint8, device="cuda")
+        r, z = buf[0, ro:ro + 4 * g.n], buf[1, zo:zo + 4 * g.n]
+        r.copy_(raw)
+        assert lib.thermal_precond_apply(g.handle, 1e-4, C.byref(opts), C.c_void_p(r.data_ptr()),
+                                         C.c_void_p(z.data_ptr()), None) == 0
+        torch.cuda.synchronize()
+        assert torch.equal(z, z0.view(torch.uint8)) and torch.equal(r, raw), (ro, zo)
