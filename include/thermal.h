@@ -244,7 +244,8 @@ th_status thermal_csr_spmv(thermal_grid* g, int variant, int precision, double d
  * z = M^{-1} r for the preconditioner selected by opts (precond, cheb_degree,
  * cheb_scaled, lanczos_steps), in FP32 (r, z: device float, n_cells).  For
  * TH_PC_CHEB the spectral interval is estimated first (cached per grid and dt), unless
- * opts->cheb_lam_min / cheb_lam_max fix it.
+ * opts->cheb_lam_min / cheb_lam_max fix it.  TH_ECUDA when a bounded wait of its kernels
+ * ran out: z is then incomplete.
  */
 th_status thermal_precond_apply(thermal_grid* g, double dt, const thermal_solve_opts* opts,
                                 const float* r, float* z, void* stream);

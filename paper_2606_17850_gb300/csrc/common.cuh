@@ -102,6 +102,25 @@ struct Ctl {
   double ad_rtrue_prev; // ||b - A x|| at the previous criterion evaluation (0: none)
 };
 
+// The control block as it is allocated: behind it the address of a pinned host word, which
+// a lost wait sets as well, so that a call that reads nothing else of the block (one
+// application of a preconditioner) learns of it at its synchronisation, without a copy
+// (one costs such a call 4 to 8 us of 30 to 130).
+struct CtlBox {
+  Ctl ctl;
+  int* wait_lost;
+};
+
+// A bounded wait ran out: record TH_ECUDA, unless an error is recorded already, and end
+// the solve's loops.  Any thread of any block, any number of times.
+__device__ __forceinline__ void ctl_wait_lost(Ctl* ctl) {
+  *(volatile int*)reinterpret_cast<CtlBox*>(ctl)->wait_lost = 1;
+  atomicCAS(&ctl->status, 0, 3);
+  ctl->outer_done = 1;
+  __threadfence();
+  atomicExch(&ctl->done, 1);
+}
+
 // Start of every kernel of the solve chains (host side: th_launch).  They are launched
 // with programmatic serialisation: a kernel's blocks may become resident while the one
 // before it finishes, so the launch itself is off the critical path; the wait returns

@@ -566,13 +566,18 @@ th_status grid_ensure_workspace(thermal_grid* g, bool need64, cudaStream_t s) {
     TH_TRY(dalloc(&g->partials, (size_t)4 * g->partials_stride + 64));
     TH_TRY(dalloc(&g->counters, 64));
     TH_CUDA(cudaMemsetAsync(g->counters, 0, 64 * sizeof(unsigned), s));
-    TH_TRY(dalloc(&g->ctl, 1));
+    CtlBox* box = nullptr;
+    TH_TRY(dalloc(&box, 1));
+    g->ctl = &box->ctl;
     TH_CUDA(cudaMemsetAsync(g->ctl, 0, sizeof(Ctl), s));
     TH_TRY(dalloc(&g->lz, 4096));
-    if (cudaMallocHost((void**)&g->ctl_host, sizeof(Ctl)) != cudaSuccess) {
+    if (cudaMallocHost((void**)&g->ctl_host, sizeof(CtlBox)) != cudaSuccess) {
       cudaGetLastError();
       return th_fail(TH_ENOMEM, "cudaMallocHost for the control block failed");
     }
+    g->wait_lost = (int*)&((CtlBox*)g->ctl_host)->wait_lost;  // the word stands where the device has its address
+    *g->wait_lost = 0;
+    TH_CUDA(cudaMemcpyAsync(&box->wait_lost, &g->wait_lost, sizeof(int*), cudaMemcpyHostToDevice, s));
     g->ws32 = true;
   }
   if (need64 && !g->ws64) {

@@ -150,6 +150,7 @@ struct thermal_grid {
   unsigned* counters = nullptr; // reduction counters (zeroed)
   Ctl* ctl = nullptr;           // device control block
   Ctl* ctl_host = nullptr;      // pinned mirror
+  int* wait_lost = nullptr;     // in the same pinned block: see CtlBox
   double* lz = nullptr;         // Lanczos alpha/beta arrays (device)
   // staging for host pointers
   void* stage_p = nullptr;

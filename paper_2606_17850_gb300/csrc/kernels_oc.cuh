@@ -441,12 +441,9 @@ __global__ void __launch_bounds__(TB_EX * EY, 1)
       for (int k = 0; k < LP; ++k) rs_[k * PL] = za[k];
     }
   }
-  if (!ok) {  // a wait ran out: record the error and end the solve's loops
+  if (!ok) {  // a wait ran out
     if (tid == 0) {
-      atomicCAS(&ctl->status, 0, 3);  // TH_ECUDA, unless an error is recorded already
-      ctl->outer_done = 1;
-      __threadfence();
-      atomicExch(&ctl->done, 1);
+      ctl_wait_lost(ctl);
       // numbers that this launch cannot have used, so that no later one meets its words
       oc_put(sync + 2 * cap, epoch0 + 0x40000000u, sums0 + 0x40000000u);
     }

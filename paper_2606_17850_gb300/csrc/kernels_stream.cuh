@@ -263,12 +263,7 @@ __global__ void __launch_bounds__(32, LMAX <= 4 ? 14 : (LMAX <= 6 ? 10 : 8))
       shift();
     }
   }
-  if (!ok && lane == 0) {  // a wait ran out: record the error and end the solve's loops
-    atomicCAS(&ctl->status, 0, 3);  // TH_ECUDA, unless an error is recorded already
-    ctl->outer_done = 1;
-    __threadfence();
-    atomicExch(&ctl->done, 1);
-  }
+  if (!ok && lane == 0) ctl_wait_lost(ctl);
   // never leave while copies into this block's shared memory are in flight
   for (int q = ok ? it : lost; q < min(ii, nit); ++q) tb_mbar_wait(bar + q % NZ, (unsigned)(q / NZ) & 1u);
   if (!LAST || done) return;

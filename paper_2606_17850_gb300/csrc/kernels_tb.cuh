@@ -197,10 +197,7 @@ __global__ void __launch_bounds__(TB_EX * EY, 1)
       // into its shared memory may still be in flight.  No later copy was issued.
       if (tid == 0) {
         tb_mbar_wait(bar, parity);
-        atomicCAS(&ctl->status, 0, 3);  // TH_ECUDA, unless an error is recorded already
-        ctl->outer_done = 1;
-        __threadfence();
-        atomicExch(&ctl->done, 1);
+        ctl_wait_lost(ctl);
       }
       break;
     }
@@ -413,10 +410,7 @@ __global__ void __launch_bounds__(TB_EX * TBF_EY, 1)
       // for this tile's copies before the CTA leaves
       if (tid == 0) {
         tb_mbar_wait(bar, parity);
-        atomicCAS(&ctl->status, 0, 3);
-        ctl->outer_done = 1;
-        __threadfence();
-        atomicExch(&ctl->done, 1);
+        ctl_wait_lost(ctl);
       }
       break;
     }

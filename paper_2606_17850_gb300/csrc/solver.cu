@@ -1649,6 +1649,15 @@ extern "C" th_status thermal_spectral_bounds(thermal_grid* g, double dt, const t
   ABI_END
 }
 
+// Ends an application: waits for it and reports a wait of its kernels that ran out (z is
+// then incomplete).
+static th_status precond_finish(thermal_grid* g, cudaStream_t s) {
+  TH_CUDA(cudaStreamSynchronize(s));
+  if (!*(volatile int*)g->wait_lost) return TH_OK;
+  return th_fail(TH_ECUDA, "device wait timed out: a bounded wait for staged or exchanged data of the preconditioner "
+                           "ran out");
+}
+
 extern "C" th_status thermal_precond_apply(thermal_grid* g, double dt, const thermal_solve_opts* opts, const float* r,
                                            float* z, void* stream) {
   ABI_BEGIN
@@ -1664,10 +1673,10 @@ extern "C" th_status thermal_precond_apply(thermal_grid* g, double dt, const the
   const BufRange br = buffer_range(r, g->device), bz = buffer_range(z, g->device);
   const int direct = th_direct_buffers(&br, &bz, sizeof(float) * (size_t)g->n, g->device);
   TH_TRY(make_plan(g, dt, &o, TH_F32, dt > 0.0, P, s, direct > 0));
+  *(volatile int*)g->wait_lost = 0;
   if (P.oc && direct) {  // one launch from r to z
     TH_TRY(oc_enqueue(P, s, 0, r, z));
-    TH_CUDA(cudaStreamSynchronize(s));
-    return TH_OK;
+    return precond_finish(g, s);
   }
   const CtlInit ci = ctl_init(&o, 1, 1, 1);
   k_ctl_reset<<<1, 1, 0, s>>>(g->ctl, ci);
@@ -1683,16 +1692,14 @@ extern "C" th_status thermal_precond_apply(thermal_grid* g, double dt, const the
     if (P.pc == TH_PC_CHEB && P.zfin == 3) V.mu = z;
     else V.zc[P.pc == TH_PC_CHEB ? P.zfin : 0] = z;
     TH_TRY(enq_precond_tail<float>(P, V, s));
-    TH_CUDA(cudaStreamSynchronize(s));
-    return TH_OK;
+    return precond_finish(g, s);
   }
   const size_t bytes = sizeof(float) * (size_t)g->n;
   TH_CUDA(cudaMemcpyAsync(g->r32, r, bytes, cudaMemcpyDeviceToDevice, s));
   TH_TRY((enq_update<float, true>(P, V, s, 0, 1, 0)));
   TH_TRY(enq_precond_tail<float>(P, V, s));
   TH_CUDA(cudaMemcpyAsync(z, z_final(P, V), bytes, cudaMemcpyDeviceToDevice, s));
-  TH_CUDA(cudaStreamSynchronize(s));
-  return TH_OK;
+  return precond_finish(g, s);
   ABI_END
 }
 

@@ -111,3 +111,45 @@ def test_fused_kernel_wait_expiry_reported(graph, kind):
     assert "timed out" in str(e.value)
     torch.cuda.synchronize()   # the context is still usable
     _normal_solve_matches_oracle(g, nx, ny, st, precision="mixed", cheb_degree=12, cheb_fuse=4, use_graph=graph)
+
+
+@pytest.mark.parametrize("nx,ny,mk,kmap,fuse", [
+    (77, 37, "c2", 0, 0),      # on chip, difference form
+    (64, 40, "c1", 0, 0),      # on chip, expanded form
+    (76, 37, "c2", 0, 4),      # tiles, layer table
+    (76, 36, "mol", 0, 3),     # tiles of 10 layers
+    (76, 37, "c2", 1, 0),      # tiles, per-face arrays
+    (772, 771, "c2", 0, 0),    # streams
+    (448, 451, "c1", 0, 0),
+])
+@pytest.mark.parametrize("inplace", [0, 1])
+def test_precond_wait_expiry_reported(nx, ny, mk, kmap, fuse, inplace):
+    """An application whose bounded wait runs out returns TH_ECUDA, through the caller's
+    buffers and through copies (z = r); the next one on the grid is the one before."""
+    import ctypes as C
+    from paper_2606_17850_gb300 import ThermalError, _lib, api
+    st = {"c1": ti.stack_c1, "c2": ti.stack_c2, "mol": ti.stack_mol}[mk]()
+    g = _grid(nx, ny, st)
+    if kmap:
+        rng = np.random.default_rng(3)
+        kc = np.repeat(np.asarray(st.k(), dtype=np.float64), nx * ny) * rng.uniform(0.5, 2.0, g.n)
+        g.set_conductivity_map(torch.from_numpy(kc).cuda())
+    r0 = torch.from_numpy(ti.random_vector(g.n, 31).astype(np.float32)).cuda()
+    o = dict(precond="cheb", cheb_degree=12, cheb_fuse=fuse)
+    z0 = g.precond(r0, 1e-4, **o)
+
+    def apply(**kw):
+        r = r0.clone()
+        z = r if inplace else torch.empty_like(r)
+        opts = api.make_opts(**o, **kw)
+        _lib.check(_lib.load().thermal_precond_apply(g.handle, 1e-4, C.byref(opts), C.c_void_p(r.data_ptr()),
+                                                     C.c_void_p(z.data_ptr()), None))
+        return z
+
+    with pytest.raises(ThermalError) as e:
+        apply(test_wait_expire=1)
+    assert e.value.status == 3 and "timed out" in str(e.value)
+    torch.cuda.synchronize()   # the context is still usable
+    assert torch.equal(apply(), z0)
+    r0[5] = float("nan")
+    apply()                    # not an error of the application
