@@ -106,28 +106,31 @@ bool is_device_pointer(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Managed memory counts as memory of the device that asks.
+// One driver query for all of it (the runtime's and the address range's one after the
+// other: an application on 64 x 64 x 8 at degree 2 31.5 instead of 29.6 us).  Managed memory
+// counts as memory of the device that asks.
 BufRange buffer_range(const void* p, int device) {
-  BufRange b{(uintptr_t)p, -1, 0, 0};
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-    cudaGetLastError();
-    return b;
-  }
-  if (a.type != cudaMemoryTypeDevice && a.type != cudaMemoryTypeManaged) return b;
-  static const PFN_cuMemGetAddressRange_v3020 range = [] {
+  static const PFN_cuPointerGetAttributes_v7000 query = [] {
     void* f = nullptr;
     cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 3020, cudaEnableDefault, &q) != cudaSuccess) {
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 7000, cudaEnableDefault, &q) != cudaSuccess) {
       cudaGetLastError();
       f = nullptr;
     }
-    return (PFN_cuMemGetAddressRange_v3020)f;
+    return (PFN_cuPointerGetAttributes_v7000)f;
   }();
+  BufRange b{(uintptr_t)p, -1, 0, 0};
+  unsigned type = 0;
+  int managed = 0, ordinal = -1;
   CUdeviceptr base = 0;
   size_t size = 0;
-  if (!range || range(&base, &size, (CUdeviceptr)p) != CUDA_SUCCESS) return b;
-  b.device = a.type == cudaMemoryTypeManaged ? device : a.device;
+  CUpointer_attribute at[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                               CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                               CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* out[5] = {&type, &managed, &ordinal, &base, &size};
+  if (!query || query(5, at, out, (CUdeviceptr)p) != CUDA_SUCCESS) return b;
+  if (!managed && type != CU_MEMORYTYPE_DEVICE) return b;
+  b.device = managed ? device : ordinal;
   b.base = (uintptr_t)base;
   b.size = size;
   return b;
