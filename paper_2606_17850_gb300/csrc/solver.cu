@@ -361,8 +361,11 @@ static th_status make_plan(thermal_grid* g, double dt, const thermal_solve_opts*
   P.v4 = (g->nx % 4 == 0);
   P.uni = g->uniform;
   // a grid whose tiles fit the SMs keeps the inner PCG on chip (any nx); an explicit
-  // cheb_fuse asks for the tile kernels
-  if (P.pc == TH_PC_CHEB && P.prec != TH_PREC_FP64 && !P.ad && P.scaled && P.uni && o->cheb_fuse == 0) {
+  // cheb_fuse asks for the chunk kernels (tiles or streams).  All three read the layer
+  // table; where nx % 4 != 0 a caller who asks for BF16 coefficients gets them, one step
+  // per launch.
+  if (P.pc == TH_PC_CHEB && (P.prec == TH_PREC_MIXED_IR || (P.prec == TH_PREC_MIXED_IR_BF16 && P.v4)) && P.scaled &&
+      P.uni && o->cheb_fuse == 0) {
     P.oc_tile = oc_shape(g->nx, g->ny, g->L, P.k);
     P.oc = P.oc_tile.rows > 0;
   }

@@ -1226,3 +1226,16 @@ def test_precond_buffers_at_any_byte(nx, ny, pc, k):
                                          C.c_void_p(z.data_ptr()), None) == 0
         torch.cuda.synchronize()
         assert torch.equal(z, z0.view(torch.uint8)) and torch.equal(r, raw), (ro, zo)
+
+
+@pytest.mark.parametrize("nx,ny,mk,k", [(37, 21, "c1", 9), (131, 37, "l7", 13), (5, 3, "c2", 2)])
+def test_bf16_coefficients_read_where_nx_is_ragged(nx, ny, mk, k):
+    """"mixed_bf16" on nx % 4 != 0: the default application reads the BF16 coefficients, as
+    one step per launch does, and is not the FP32 one."""
+    g = grid_of(nx, ny, STACKS[mk]())
+    r = cuda(ti.random_vector(g.n, 5).astype(np.float32))
+    for dt in (0.0, 1e-4):
+        z = g.precond(r, dt, precision="mixed_bf16", precond="cheb", cheb_degree=k)
+        assert torch.equal(z, g.precond(r, dt, precision="mixed_bf16", precond="cheb", cheb_degree=k, cheb_fuse=1))
+        z32 = g.precond(r, dt, precision="mixed", precond="cheb", cheb_degree=k)
+        assert (z - z32).abs().max().item() > 1e-5 * z32.abs().max().item()
