@@ -16,6 +16,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "sums.cuh"
+
 #define TH_MAXL 32            // maximum number of layers
 #define TH_BX 32              // threads per block along x
 #define TH_BY 8               // threads per block along y
@@ -311,6 +313,12 @@ __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+// the products of a column's layer pairs
+template <int LP>
+__device__ __forceinline__ float pair_sum(float2 (&t)[LP]) {
+  tree_sum(t, [](const float2& a, const float2& b) { return __fadd2_rn(a, b); });
+  return t[0].x + t[0].y;
 }
 __device__ __forceinline__ double warp_max(double v) {
 #pragma unroll

@@ -128,7 +128,7 @@ __device__ __forceinline__ bool oc_recv(const OCWord* w, long long stride, float
 
 // scalars of the iteration, decided by thread 0 of every CTA from the same totals
 struct OCShared {
-  double red[32];
+  float red[32 * 16];
   double rz, rr0, tgt;
   float alpha, beta;
   int it, status, stop, ok;
@@ -139,17 +139,28 @@ constexpr size_t oc_smem_bytes() {
   return (size_t)(2 + 3) * (LMAX / 2) * EY * TB_EX * sizeof(float2);
 }
 
-// A float per thread summed over the grid and handed to fin(total) in thread 0 of every
-// CTA.  False when the wait ran out.
-template <typename F>
+// A float per thread, the sum of a column's LP layer pairs, summed over the grid and handed
+// to fin(total) in thread 0 of every CTA.  False when the wait ran out.  A product meets at
+// most five FP32 additions, those of its column among them, as in the one-step kernels
+// (one cell a thread, 32 lanes); the rest keeps its rounding errors.  As fast as a plain
+// FP32 sum of column and lanes (steady 64 x 64 x 4 757 us with it, 755 now); all five lane
+// steps with their errors kept took 791.
+template <int LP, typename F>
 __device__ __forceinline__ bool oc_sum(OCShared& sh, OCWord* sync, int cap, unsigned& sums, float v, F fin) {
+  constexpr int FP = 5 - (tree_depth(LP) + 1), G = 32 >> FP;  // lane steps in FP32, values left of a warp
+  static_assert(FP >= 1 && G <= 16, "lane groups of a column sum");
   const int t = thread_linear_id(), nw = block_threads() >> 5, nblk = gridDim.x;
   const unsigned epoch = ++sums;
-  v = warp_sum(v);
-  if ((t & 31) == 0) sh.red[t >> 5] = (double)v;
+#pragma unroll
+  for (int o = 1; o < (1 << FP); o *= 2) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((t & ((1 << FP) - 1)) == 0) sh.red[t >> FP] = v;
   __syncthreads();
   if (t < 32) {
-    const double mine = warp_sum(t < nw ? sh.red[t] : 0.0);
+    Sum2 part{0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < G; ++i)
+      if (t + 32 * i < nw * G) sum2_add(part, sh.red[t + 32 * i]);
+    const double mine = warp_sum(sum2_value(part));
     OCWord* set = sync + (size_t)(epoch & 1u) * cap;
     if (t == 0) oc_put(set + blockIdx.x, (unsigned long long)__double_as_longlong(mine), epoch);
     double tot = 0.0;
@@ -341,22 +352,20 @@ __global__ void __launch_bounds__(TB_EX * EY, 1)
         }
       }
       // nobody may record the last number before everybody has read the first
-      if (epoch != epoch0) ok = oc_sum(sh, sync, cap, sums, 0.f, [](double) {});
+      if (epoch != epoch0) ok = oc_sum<LP>(sh, sync, cap, sums, 0.f, [](double) {});
       break;
     }
     // ---- r^T z, beta, p = z + beta p on the interior and the ring around it
     float part = 0.f;
     ++epoch;
     if (interior) {
+      float2 t[LP];
 #pragma unroll
-      for (int k = 0; k < LP; ++k) {
-        const float2 rv = rs_[k * PL];
-        part += rv.x * za[k].x;
-        part += rv.y * za[k].y;
-      }
+      for (int k = 0; k < LP; ++k) t[k] = __fmul2_rn(rs_[k * PL], za[k]);
+      part = pair_sum(t);
       if (pub1) oc_send<LP>(col0 + (epoch & 1u) * set1, d.pxy, za, za, epoch);
     }
-    ok = oc_sum(sh, sync, cap, sums, part, [&](double t) {
+    ok = oc_sum<LP>(sh, sync, cap, sums, part, [&](double t) {
       sh.beta = (sh.it == 0 || !(sh.rz != 0.0)) ? 0.f : (float)(t / sh.rz);
       sh.rz = t;
     });
@@ -377,6 +386,7 @@ __global__ void __launch_bounds__(TB_EX * EY, 1)
     // ---- mu = A p in difference form (kept in zb), p^T mu
     part = 0.f;
     if (interior) {
+      float2 t[LP];
 #pragma unroll
       for (int k = 0; k < LP; ++k) {
         const float2* q = pl + k * PL;
@@ -392,11 +402,11 @@ __global__ void __launch_bounds__(TB_EX * EY, 1)
         a = __ffma2_rn(P.gzu[k], dif(up), a);  // the faces at the ends are 0
         a = __ffma2_rn(P.gzd[k], dif(dn), a);
         zb[k] = a;
-        part += v.x * a.x;
-        part += v.y * a.y;
+        t[k] = __fmul2_rn(v, a);
       }
+      part = pair_sum(t);
     }
-    ok = oc_sum(sh, sync, cap, sums, part, [&](double pAp) {
+    ok = oc_sum<LP>(sh, sync, cap, sums, part, [&](double pAp) {
       const bool fine = pAp > 0.0 && sh.rz > 0.0;
       sh.alpha = fine ? (float)(sh.rz / pAp) : 0.f;
       if (!fine) {  // breakdown (see fin_pap)
@@ -410,6 +420,7 @@ __global__ void __launch_bounds__(TB_EX * EY, 1)
     part = 0.f;
     ++epoch;
     if (interior) {
+      float2 t[LP];
 #pragma unroll
       for (int k = 0; k < LP; ++k) {
         const float2 p = ps_[k * PL], x = xs_[k * PL], mu = zb[k];
@@ -419,12 +430,12 @@ __global__ void __launch_bounds__(TB_EX * EY, 1)
         rv.y -= alpha * mu.y;
         rs_[k * PL] = rv;
         za[k] = rv;
-        part += rv.x * rv.x;
-        part += rv.y * rv.y;
+        t[k] = __fmul2_rn(rv, rv);
       }
+      part = pair_sum(t);
       if (pubH) oc_send<LP>(col0 + (epoch & 1u) * set1, d.pxy, za, za, epoch);
     }
-    ok = oc_sum(sh, sync, cap, sums, part, [&](double rr) {
+    ok = oc_sum<LP>(sh, sync, cap, sums, part, [&](double rr) {
       sh.it += 1;
       sh.rr0 = rr;  // from here on the current ||r||^2
       if (!isfinite(rr)) {
