@@ -314,6 +314,13 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+// with the errors of the lane steps kept as well
+__device__ __forceinline__ double warp_sum(Sum2 v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    sum2_add(v, Sum2{__shfl_xor_sync(0xffffffffu, v.s, o), __shfl_xor_sync(0xffffffffu, v.e, o)});
+  return sum2_value(v);
+}
 // the products of a column's layer pairs
 template <int LP>
 __device__ __forceinline__ float pair_sum(float2 (&t)[LP]) {
@@ -388,8 +395,8 @@ template <typename TA> __device__ __forceinline__ TA lay_s(const LayerTab* t, in
 template <> __device__ __forceinline__ double lay_s<double>(const LayerTab* t, int z) { return __ldg(&t->s64[z]); }
 template <> __device__ __forceinline__ float lay_s<float>(const LayerTab* t, int z) { return __ldg(&t->s32[z]); }
 
-// Sum NQ per-thread values (type T, warp level in T) over the block, then over the
-// grid: each block writes one FP64 partial; the last block sums the partials in a
+// Sum NQ per-thread values (type T: float, double or Sum2; warp level in T) over the block,
+// then over the grid: each block writes one FP64 partial; the last block sums the partials in a
 // fixed order.  Returns true in thread 0 of the last block, with tot[] valid there.
 template <typename T, int NQ>
 __device__ __forceinline__ bool grid_reduce(T (&v)[NQ], double* partials, int stride, unsigned* counter,
@@ -399,10 +406,9 @@ __device__ __forceinline__ bool grid_reduce(T (&v)[NQ], double* partials, int st
   const int t = thread_linear_id();
   const int nw = (block_threads() + 31) >> 5;
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) v[q] = warp_sum(v[q]);
-  if ((t & 31) == 0) {
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) sm[q][t >> 5] = (double)v[q];
+  for (int q = 0; q < NQ; ++q) {
+    const double w = (double)warp_sum(v[q]);
+    if ((t & 31) == 0) sm[q][t >> 5] = w;
   }
   __syncthreads();
   if (t == 0) {

@@ -139,7 +139,8 @@ __device__ __forceinline__ void mgt_down(const MGDev& v, const MGUni<LMAX>& U, i
 }
 
 // Way up: x = x_in + P x_c, x_out = x + omega T^-1 (b - A x).  With RZ it returns this
-// thread's part of b^T x_out (b read again, so that the sweep can reuse its registers).
+// thread's part of b^T x_out, its layers' products added as a tree (b read again, so that
+// the sweep can reuse its registers; the products take the places of what is used up).
 template <int LMAX, bool UNI, int EY, bool CG, bool RZ>
 __device__ __forceinline__ float mgt_up(const MGDev& v, const MGUni<LMAX>& U, int bx, int by, const float* b,
                                         const float* xin, const float* xc, int nxc, int nyc, float* xout, float* xs) {
@@ -163,7 +164,7 @@ __device__ __forceinline__ float mgt_up(const MGDev& v, const MGUni<LMAX>& U, in
 #pragma unroll
   for (int z = 0; z < LMAX; ++z) bv[z] = (p.inner && z < L) ? mgt_ld<CG>(b + p.i0 + p.pxy * z) : 0.f;
   __syncthreads();
-  float rz = 0.f, dprev = 0.f;
+  float dprev = 0.f;
 #pragma unroll
   for (int z = 0; z < LMAX; ++z) {
     const float res = mgt_residual<LMAX, UNI, EY>(C, p, xs, z, bv[z], xv);
@@ -174,10 +175,11 @@ __device__ __forceinline__ float mgt_up(const MGDev& v, const MGUni<LMAX>& U, in
   for (int z = LMAX - 1; z >= 0; --z) {
     dn = bv[z] + C.w(z) * dn;
     const float o = xv[z] + kMGOmega * dn;
-    if (p.inner && z < L) {
-      xout[p.i0 + p.pxy * z] = o;
-      if (RZ) rz += mgt_ld<CG>(b + p.i0 + p.pxy * z) * o;
-    }
+    const bool on = p.inner && z < L;
+    if (on) xout[p.i0 + p.pxy * z] = o;
+    if (RZ) bv[z] = on ? mgt_ld<CG>(b + p.i0 + p.pxy * z) * o : 0.f;
   }
-  return rz;
+  if (!RZ) return 0.f;
+  tree_sum(bv, [](float u, float w) { return u + w; });
+  return bv[0];
 }

@@ -161,15 +161,16 @@ __global__ void __launch_bounds__(MGT_EX* MG_EY, LMAX <= 12 ? MG_MINB : 1)
     return;
   }
   // the tiles over the blocks that are resident at once, so that the reduction's tail (7 us
-  // of 19 with one tile per block at 512 x 512 x 8) is paid once per block
-  float part[1] = {0.f};
+  // of 19 with one tile per block at 512 x 512 x 8) is paid once per block; a thread's sum
+  // over its tiles keeps its rounding errors
+  Sum2 part[1] = {{0.f, 0.f}};
   const int tx = (v.nx + MGT_EX - 3) / (MGT_EX - 2);
   for (int q = blockIdx.x; q < mgt_tiles<MG_EY>(v.nx, v.ny); q += gridDim.x) {
-    part[0] += mgt_up<LMAX, UNI, MG_EY, false, RZ>(v, U, q % tx, q / tx, b, xin, xc, nxc, nyc, xout, mg_xs);
+    sum2_add(part[0], mgt_up<LMAX, UNI, MG_EY, false, RZ>(v, U, q % tx, q / tx, b, xin, xc, nxc, nyc, xout, mg_xs));
     __syncthreads();
   }
   double tot[1];
-  if (!grid_reduce<float, 1>(part, partials, stride, counter, tot)) return;
+  if (!grid_reduce<Sum2, 1>(part, partials, stride, counter, tot)) return;
   ctl->rz_next = tot[0];
   ctl_set_beta(ctl);
 }
@@ -194,7 +195,7 @@ __global__ void __launch_bounds__(MGT_EX* MG_EY, 1)
     for (int i = t; i < (int)(sizeof(MGCLev<LMAX>) / 4) * (nl - k0); i += MGT_EX * MG_EY) dst[i] = __ldg(src + i);
   }
   if (__syncthreads_or(t == 0 && ld_int(&ctl->done))) return;  // set by an earlier kernel: every block sees it
-  float part[1] = {0.f};
+  Sum2 part[1] = {{0.f, 0.f}};
   for (int k = k0; k + 1 < nl; ++k) {
     const MGCLev<LMAX>& l = sl[k - k0];
     const int nxc = (l.nx + 1) / 2, nyc = (l.ny + 1) / 2, tx = (l.nx + MGT_EX - 3) / (MGT_EX - 2);
@@ -235,13 +236,13 @@ __global__ void __launch_bounds__(MGT_EX* MG_EY, 1)
       float rz;
       if (l.uni) rz = mgt_up<LMAX, true, MG_EY, true, true>(v, l.t, q % tx, q / tx, b, l.x, xc, nxc, nyc, out, mg_xs);
       else rz = mgt_up<LMAX, false, MG_EY, true, true>(v, l.t, q % tx, q / tx, b, l.x, xc, nxc, nyc, out, mg_xs);
-      if (k == 0) part[0] += rz;
+      if (k == 0) sum2_add(part[0], rz);
     }
     if (k > k0) mg_cluster_sync();
   }
   if (k0 != 0) return;
   double tot[1];
-  if (!grid_reduce<float, 1>(part, partials, stride, counter, tot)) return;
+  if (!grid_reduce<Sum2, 1>(part, partials, stride, counter, tot)) return;
   ctl->rz_next = tot[0];
   ctl_set_beta(ctl);
 }

@@ -17,6 +17,11 @@ __host__ __device__ __forceinline__ void sum2_add(Sum2& a, float v) {
   a.s = t;
 }
 
+__host__ __device__ __forceinline__ void sum2_add(Sum2& a, const Sum2& o) {
+  sum2_add(a, o.s);
+  a.e += o.e;
+}
+
 // (an overflow or a NaN stays what it is in s; e is a NaN then)
 __host__ __device__ __forceinline__ double sum2_value(const Sum2& a) {
   return a.e - a.e == 0.f ? (double)a.s + (double)a.e : (double)a.s;

@@ -17,6 +17,15 @@ extern "C" double sum2(const float* v, int n) {  // one after the other, as rows
   for (int i = 0; i < n; ++i) sum2_add(a, v[i]);
   return sum2_value(a);
 }
+extern "C" double lanes(const float* v) {  // the exchange pattern of warp_sum(Sum2)
+  Sum2 a[32], b[32];
+  for (int i = 0; i < 32; ++i) a[i] = {v[i], 0.f};
+  for (int o = 16; o > 0; o >>= 1) {
+    for (int i = 0; i < 32; ++i) { b[i] = a[i]; sum2_add(b[i], a[i ^ o]); }
+    for (int i = 0; i < 32; ++i) a[i] = b[i];
+  }
+  return sum2_value(a[0]);
+}
 extern "C" int depth(int n) { return tree_depth(n); }
 template <int N> float tree(const float* v) {
   float t[N];
@@ -25,7 +34,7 @@ template <int N> float tree(const float* v) {
   return t[0];
 }
 extern "C" float trees(int n, const float* v) {
-  return n == 1 ? tree<1>(v) : n == 2 ? tree<2>(v) : n == 3 ? tree<3>(v) : n == 4 ? tree<4>(v) : tree<6>(v);
+  return n == 1 ? tree<1>(v) : n == 2 ? tree<2>(v) : n == 3 ? tree<3>(v) : n == 4 ? tree<4>(v) : n == 6 ? tree<6>(v) : tree<32>(v);
 }
 """
 
@@ -41,6 +50,7 @@ def lib(tmp_path_factory):
     lib = C.CDLL(str(d / "s.so"))
     fp = C.POINTER(C.c_float)
     lib.sum2.argtypes, lib.sum2.restype = [fp, C.c_int], C.c_double
+    lib.lanes.argtypes, lib.lanes.restype = [fp], C.c_double
     lib.trees.argtypes, lib.trees.restype = [C.c_int, fp], C.c_float
     return lib
 
@@ -69,6 +79,8 @@ def test_long_sums_keep_their_rounding_errors(lib, n):
         exact, mag = math.fsum(v.tolist()), math.fsum(np.abs(v).tolist())
         bound = (n * U) ** 2 * mag + 2.0 ** -52 * mag
         assert abs(lib.sum2(_p(v), n) - exact) <= bound, name
+        if n == 32:
+            assert abs(lib.lanes(_p(v)) - exact) <= bound, name
         if name == "small" and n >= 12:
             plain = np.float32(0)
             for x in v:
@@ -76,7 +88,7 @@ def test_long_sums_keep_their_rounding_errors(lib, n):
             assert abs(float(plain) - exact) > 100 * bound
 
 
-@pytest.mark.parametrize("n", [1, 2, 3, 4, 6])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 6, 32])
 def test_tree_of_a_column(lib, n):
     """At most ceil(log2 n) roundings on the way of any term (tree_depth)."""
     v = _sets(n)["signed"]
@@ -88,8 +100,8 @@ def test_tree_of_a_column(lib, n):
 def test_overflow_and_nan_stay(lib):
     v = np.zeros(32, np.float32)
     v[3] = v[9] = 3e38
-    assert lib.sum2(_p(v), 32) == math.inf
+    assert lib.sum2(_p(v), 32) == math.inf and lib.lanes(_p(v)) == math.inf
     v[9] = np.inf
-    assert lib.sum2(_p(v), 32) == math.inf
+    assert lib.sum2(_p(v), 32) == math.inf and lib.lanes(_p(v)) == math.inf
     v[20] = np.nan
-    assert math.isnan(lib.sum2(_p(v), 32))
+    assert math.isnan(lib.lanes(_p(v))) and math.isnan(lib.sum2(_p(v), 32))
