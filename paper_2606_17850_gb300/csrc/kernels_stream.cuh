@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(32, LMAX <= 4 ? 14 : (LMAX <= 6 ? 10 : 8))
   unsigned long long* bars = (unsigned long long*)(zp_ring + (FIRST ? 0 : NZ * ROW));
   unsigned long long* bar = bars + 1;  // bars[0]: the test hook's, never completed
   const int L = d.L, nx = d.nx, ny = d.ny;
-  float part[1] = {0.f};
+  Sum2 part[1] = {{0.f, 0.f}};  // r^T z: a row's products as a tree, the rows with their rounding errors
   if (lane == 0) {
     for (int i = 0; i < 1 + NZ; ++i) tb_mbar_init(bars + i, 1);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -225,14 +225,13 @@ __global__ void __launch_bounds__(32, LMAX <= 4 ? 14 : (LMAX <= 6 ? 10 : 8))
         for (int z = 0; z < LMAX; ++z) {
           if (z < L) {
             *(float2*)((char*)(out_cur + d.pxy * z) + off) = out[z];
-            if (LAST) {
-              const float2 rv = rq[z * (ST_BW / 2)];
-              part[0] += rv.x * out[z].x;
-              part[0] += rv.y * out[z].y;
-            } else {
-              *(float2*)((char*)(out_prev + d.pxy * z) + off) = Z[S - 1][M][z];
-            }
+            if (!LAST) *(float2*)((char*)(out_prev + d.pxy * z) + off) = Z[S - 1][M][z];
           }
+        }
+        if (LAST) {  // (layers beyond the stack's are zeros)
+#pragma unroll
+          for (int z = 0; z < LMAX; ++z) out[z] = __fmul2_rn(rq[z * (ST_BW / 2)], out[z]);
+          sum2_add(part[0], pair_sum(out));
         }
       }
     }
@@ -268,7 +267,7 @@ __global__ void __launch_bounds__(32, LMAX <= 4 ? 14 : (LMAX <= 6 ? 10 : 8))
   for (int q = ok ? it : lost; q < min(ii, nit); ++q) tb_mbar_wait(bar + q % NZ, (unsigned)(q / NZ) & 1u);
   if (!LAST || done) return;
   double tot[1];
-  if (!grid_reduce<float, 1>(part, partials, stride, counter, tot)) return;
+  if (!grid_reduce<Sum2, 1>(part, partials, stride, counter, tot)) return;
   ctl->rz_next = tot[0];
   ctl_set_beta(ctl);
 }
