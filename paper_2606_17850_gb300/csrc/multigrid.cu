@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(MGT_EX* MG_EY, LMAX <= 12 ? MG_MINB : 1)
               float* __restrict__ x, int nxc, int nyc, float* __restrict__ bc) {
   grid_dep_enter();
   if (ld_int(&ctl->done)) return;
-  extern __shared__ float mg_xs[];
+  extern __shared__ __align__(16) float mg_xs[];
   mgt_down<LMAX, UNI, MG_EY, false>(v, U, blockIdx.x, blockIdx.y, b, x, nxc, nyc, bc, mg_xs);
 }
 
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(MGT_EX* MG_EY, LMAX <= 12 ? MG_MINB : 1)
             double* partials, int stride, unsigned* counter) {
   grid_dep_enter();
   if (ld_int(&ctl->done)) return;
-  extern __shared__ float mg_xs[];
+  extern __shared__ __align__(16) float mg_xs[];
   if (!RZ) {
     mgt_up<LMAX, UNI, MG_EY, false, RZ>(v, U, blockIdx.x, blockIdx.y, b, xin, xc, nxc, nyc, xout, mg_xs);
     return;
@@ -186,7 +186,8 @@ __global__ void __launch_bounds__(MGT_EX* MG_EY, 1)
     k_mg_levels(Ctl* ctl, const MGCLev<LMAX>* lv, int L, int k0, int nl, int nc, const float* __restrict__ cinv,
                 const float* b0, float* z, double* partials, int stride, unsigned* counter) {
   grid_dep_enter();
-  extern __shared__ float mg_xs[];
+  extern __shared__ __align__(16) float mg_xs[];
+  static_assert(alignof(MGCLev<LMAX>) <= 16 && mg_xs_bytes<LMAX>() % 16 == 0, "descriptors behind the tile");
   MGCLev<LMAX>* sl = reinterpret_cast<MGCLev<LMAX>*>(mg_xs + LMAX * MGT_EX * MG_EY);  // levels k0 ..
   const int t = thread_linear_id();
   {

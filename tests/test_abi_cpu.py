@@ -182,3 +182,19 @@ def test_precond_buffers_read_in_place_only_where_kernels_can(lib):
     assert ask(r=(0, 0, 4 * n), z=(n - 16, 0, 4 * n), **same) == 0
     assert ask(r=(n - 4, 0, 4 * n), z=(0, 0, 4 * n), **same) == 0
     assert ask(r=(0, 0, 4 * n), z=(n, 0, 4 * n), **same) == 2
+
+
+def test_dynamic_shared_memory_states_its_alignment():
+    """A kernel that places structs in its dynamic shared memory declares the alignment they
+    need: the element type alone promises that of a float."""
+    import glob
+    csrc = os.path.join(ROOT, "paper_2606_17850_gb300", "csrc")
+    cast = 0
+    for f in sorted(glob.glob(os.path.join(csrc, "*.cu*"))):
+        text = open(f).read()
+        for quals, name in re.findall(r"extern __shared__ ([^;]*?)(\w+)\[\];", text):
+            if re.search(r"reinterpret_cast<(?!const (?:int|float))[^>]*[^)]*>\(\s*%s\b" % name, text):
+                cast += 1
+                m = re.search(r"__align__\((\d+)\)", quals)
+                assert m and int(m.group(1)) >= 16, (os.path.basename(f), name)
+    assert cast > 0
