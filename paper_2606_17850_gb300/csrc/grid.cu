@@ -331,8 +331,11 @@ dim3 grid_blocks(const thermal_grid* g) {
   return dim3((g->nx + TH_BX - 1) / TH_BX, (g->ny + TH_BY - 1) / TH_BY, g->L);
 }
 
+// (an array that is there already stays: a call that failed half way through its
+// allocations leaves the first ones for the next)
 template <typename T>
 static th_status dalloc(T** p, size_t n) {
+  if (*p) return TH_OK;
   cudaError_t e = cudaMalloc((void**)p, sizeof(T) * (n ? n : 1));
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -416,12 +419,10 @@ th_status grid_ensure_tab(thermal_grid* g, double dt, cudaStream_t s) {
   if (dt > 0.0 && !g->has_c) return th_fail(TH_ESTATE, "grid was created without heat capacities");
   const double key = dt > 0.0 ? dt : 0.0;
   if (g->tab_valid && g->tab_dt == key) return TH_OK;
-  if (!g->tab) TH_TRY(dalloc(&g->tab, 1));
-  if (!g->invd32) {
-    TH_TRY(dalloc(&g->invd32, g->n));
-    TH_TRY(dalloc(&g->invd64, g->n));
-    TH_TRY(dalloc(&g->isqd32, g->n));
-  }
+  TH_TRY(dalloc(&g->tab, 1));
+  TH_TRY(dalloc(&g->invd32, g->n));
+  TH_TRY(dalloc(&g->invd64, g->n));
+  TH_TRY(dalloc(&g->isqd32, g->n));
   std::memset(&g->tab_host, 0, sizeof(LayerTab));
   const double S = g->dx * g->dy;
   for (int l = 0; l < g->L; ++l) {
@@ -491,14 +492,12 @@ th_status grid_ensure_qd(thermal_grid* g, double dt, cudaStream_t s) {
   TH_TRY(grid_ensure_tab(g, dt, s));
   const double key = dt > 0.0 ? dt : 0.0;
   if (g->qd_valid && g->qd_dt == key) return TH_OK;
-  if (!g->qd4) {
-    TH_TRY(dalloc(&g->qd4, g->n));
-    TH_TRY(dalloc(&g->qd5, g->n));
-    TH_TRY(dalloc(&g->qd6, g->n));
-    TH_TRY(dalloc(&g->qd7, g->n));
-    TH_TRY(dalloc(&g->diag32, g->n));
-    TH_TRY(dalloc(&g->diag64, g->n));
-  }
+  TH_TRY(dalloc(&g->qd4, g->n));
+  TH_TRY(dalloc(&g->qd5, g->n));
+  TH_TRY(dalloc(&g->qd6, g->n));
+  TH_TRY(dalloc(&g->qd7, g->n));
+  TH_TRY(dalloc(&g->diag32, g->n));
+  TH_TRY(dalloc(&g->diag64, g->n));
   unsigned long long* mx = nullptr;
   TH_TRY(dalloc(&mx, 1));
   unsigned long long hmx = 0;
@@ -526,7 +525,7 @@ th_status grid_ensure_dg64(thermal_grid* g, double dt, cudaStream_t s) {
   TH_TRY(grid_ensure_tab(g, dt, s));
   const double key = dt > 0.0 ? dt : 0.0;
   if (g->dg64_valid && g->dg64_dt == key) return TH_OK;
-  if (!g->dg64) TH_TRY(dalloc(&g->dg64, g->n));
+  TH_TRY(dalloc(&g->dg64, g->n));
   k_diag_out<<<grid_blocks(g), dim3(TH_BX, TH_BY), 0, s>>>(grid_dims(g), g->f64, g->tab, g->dg64);
   TH_CHECK_LAUNCH();
   g->dg64_dt = key;
@@ -537,10 +536,8 @@ th_status grid_ensure_dg64(thermal_grid* g, double dt, cudaStream_t s) {
 th_status grid_ensure_zline(thermal_grid* g, double dt, cudaStream_t s) {
   TH_TRY(grid_ensure_tab(g, dt, s));
   if (g->zl_valid) return TH_OK;
-  if (!g->zl_c) {
-    TH_TRY(dalloc(&g->zl_c, g->n));
-    TH_TRY(dalloc(&g->zl_m, g->n));
-  }
+  TH_TRY(dalloc(&g->zl_c, g->n));
+  TH_TRY(dalloc(&g->zl_m, g->n));
   dim3 b(32, 8), gr((g->nx + 31) / 32, (g->ny + 7) / 8);
   k_setup_zline<<<gr, b, 0, s>>>(grid_dims(g), g->f64, g->tab, g->zl_m, g->zl_c);
   TH_CHECK_LAUNCH();
@@ -569,13 +566,14 @@ th_status grid_ensure_workspace(thermal_grid* g, bool need64, cudaStream_t s) {
     TH_TRY(dalloc(&g->partials, (size_t)4 * g->partials_stride + 64));
     TH_TRY(dalloc(&g->counters, 64));
     TH_CUDA(cudaMemsetAsync(g->counters, 0, 64 * sizeof(unsigned), s));
-    CtlBox* box = nullptr;
+    CtlBox* box = reinterpret_cast<CtlBox*>(g->ctl);
     TH_TRY(dalloc(&box, 1));
     g->ctl = &box->ctl;
     TH_CUDA(cudaMemsetAsync(g->ctl, 0, sizeof(Ctl), s));
     TH_TRY(dalloc(&g->lz, 4096));
-    if (cudaMallocHost((void**)&g->ctl_host, sizeof(CtlBox)) != cudaSuccess) {
+    if (!g->ctl_host && cudaMallocHost((void**)&g->ctl_host, sizeof(CtlBox)) != cudaSuccess) {
       cudaGetLastError();
+      g->ctl_host = nullptr;
       return th_fail(TH_ENOMEM, "cudaMallocHost for the control block failed");
     }
     g->wait_lost = (int*)&((CtlBox*)g->ctl_host)->wait_lost;  // the word stands where the device has its address

@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <vector>
 
 #include "internal.h"
@@ -459,8 +460,9 @@ th_status grid_ensure_mg(thermal_grid* g, double dt, cudaStream_t s) {
   const double key = dt > 0.0 ? dt : 0.0;
   if (g->mg && g->mg_valid && g->mg->dt == key) return TH_OK;
   if (g->L > 32) return th_fail(TH_EINVAL, "multigrid supports at most 32 layers");
+  g->mg_valid = false;  // until the rebuild below is complete
   if (!g->mg) {
-    MGHier* h = new MGHier();
+    auto h = std::make_unique<MGHier>();  // the grid's once every level has its memory
     int nx = g->nx, ny = g->ny;
     while (true) {
       MGLevelH l;
@@ -472,7 +474,6 @@ th_status grid_ensure_mg(thermal_grid* g, double dt, cudaStream_t s) {
       nx = (nx + 1) / 2;
       ny = (ny + 1) / 2;
     }
-    g->mg = h;
     for (size_t k = 0; k < h->lv.size(); ++k) {
       MGLevelH& l = h->lv[k];
       TH_TRY(mg_alloc(&l.s, l.n));
@@ -494,6 +495,7 @@ th_status grid_ensure_mg(thermal_grid* g, double dt, cudaStream_t s) {
         TH_TRY(mg_alloc(&l.b, l.n));
       }
     }
+    g->mg = h.release();
   }
   MGHier* h = g->mg;
   const int L = g->L;
