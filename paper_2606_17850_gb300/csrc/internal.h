@@ -161,6 +161,7 @@ struct thermal_grid {
 
   GraphCache* graphs = nullptr;
   void* oc_sync = nullptr;  // exchange words of the on-chip inner PCG
+  bool oc_refused = false;  // the running call's cooperative launch was refused
   int zc_tuned = 0;  // layers per thread in the vectorised kernels (autotuned)
 
   ~thermal_grid();
@@ -227,6 +228,8 @@ void graph_cache_free(GraphCache* c);
 th_status solver_cheb_coeffs(thermal_grid* g, double dt, const thermal_solve_opts* o, std::vector<float>& c1,
                              std::vector<float>& c2, float* inv_theta, double* lmin, double* lmax, cudaStream_t s);
 int device_sms();
+// SMs that kernels launched on s can run on: fewer than the device's in a green context.
+int stream_sms(cudaStream_t s);
 // 3-D tensor map of one FP32 field (x fastest, then y, then layer) with a box of bw x bh
 // columns x L layers; cells outside the grid read as zero.  TH_EINVAL unless nx % 4 == 0
 // and the base is 16-byte aligned.
@@ -251,7 +254,7 @@ th_status cheb_stream_8(thermal_grid* g, const Dims& d, const StreamChunk& c, cu
 // pcg_oc.cu: the whole FP32 inner PCG with the Chebyshev preconditioner (solve = 1: on
 // r, the correction in d32), or one application of it (solve = 0: z = M^-1 r), as one
 // cooperative launch over tiles that stay on chip; layer-uniform grids whose tiles fit
-// the SMs (oc_shape's rows > 0).
+// the SMs of the stream (oc_shape's rows > 0).
 struct OCShape { int rows, halo; };
 struct OCRun {
   OCShape shape;
@@ -262,7 +265,8 @@ struct OCRun {
   double inv_theta;
   int expire_test;
 };
-OCShape oc_shape(int nx, int ny, int L, int k);
+OCShape oc_shape(int nx, int ny, int L, int k, int sms);
+bool oc_cannot_launch(cudaError_t e);  // the device or a partition of it has no room for the grid
 th_status oc_prepare(thermal_grid* g, cudaStream_t s);
 th_status oc_run(thermal_grid* g, const OCRun& o, cudaStream_t s);
 // FP32 / BF16-coefficient y = A x through the vectorised kernel; TH_EINVAL when nx % 4 != 0.

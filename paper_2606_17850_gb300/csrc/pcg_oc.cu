@@ -6,12 +6,12 @@
 #include "kernels_oc.cuh"
 
 // Rows of the grown tile and halo width, {0, 0} where the kernel does not apply: the tiles
-// have to fit the SMs, one each, and a tile has to hold its neighbour's halo.  Among the
+// have to fit the `sms` that the launch may use, one each, and a tile has to hold its neighbour's halo.  Among the
 // shapes that do, the one with the least time for the k - 1 steps.  Measured over 64^2 to
 // 301 x 203 columns, 16 / 24 / 32 rows and halos of 2 to 8: a step takes 5.2 ns per row and
 // layer pair of the grown tile (0.17 us at 16 rows of 4 layers, 0.67 us at 32 rows of 8),
 // an exchange 1.3 to 1.9 us whatever its width.
-OCShape oc_shape(int nx, int ny, int L, int k) {
+OCShape oc_shape(int nx, int ny, int L, int k, int sms) {
   OCShape best{0, 0};
   if (L > 12 || k < 2 || k > OC_MAXK) return best;
   const int lp = L <= 4 ? 2 : (L <= 6 ? 3 : (L <= 8 ? 4 : 6));
@@ -20,7 +20,7 @@ OCShape oc_shape(int nx, int ny, int L, int k) {
     if (L > 8 && ey == 32) continue;  // 12 layers: at most 768 threads' registers
     for (int h = 2; h <= 8 && 3 * h <= ey; ++h) {
       const long long tx = TB_EX - 2 * h, ty = ey - 2 * h;
-      if (((nx + tx - 1) / tx) * ((ny + ty - 1) / ty) > device_sms()) continue;
+      if (((nx + tx - 1) / tx) * ((ny + ty - 1) / ty) > sms) continue;
       const double t = (k - 1) * 0.0052 * lp * ey + 1.6 * ((k - 1 + h - 1) / h);
       if (t < least) {
         least = t;
@@ -29,6 +29,10 @@ OCShape oc_shape(int nx, int ny, int L, int k) {
     }
   }
   return best;
+}
+
+bool oc_cannot_launch(cudaError_t e) {
+  return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported || e == cudaErrorLaunchOutOfResources;
 }
 
 template <int LMAX, int EY, bool DIFF>
@@ -84,9 +88,12 @@ static th_status oc_launch(thermal_grid* g, const OCRun& o, cudaStream_t s) {
   c.stream = s;
   c.attrs = &at1;
   c.numAttrs = 1;
-  TH_CUDA(cudaLaunchKernelEx(&c, kern, d, ntx, o.shape.halo, o.solve, g->ctl, o.r, g->d32, o.z, prm,
-                             (OCWord*)g->oc_sync, cap));
-  return TH_OK;
+  const cudaError_t e = cudaLaunchKernelEx(&c, kern, d, ntx, o.shape.halo, o.solve, g->ctl, o.r, g->d32, o.z, prm,
+                                           (OCWord*)g->oc_sync, cap);
+  if (e == cudaSuccess) return TH_OK;
+  g->oc_refused = oc_cannot_launch(e);
+  cudaGetLastError();
+  return th_fail(TH_ECUDA, "launch of the on-chip inner solve failed: %s", cudaGetErrorString(e));
 }
 
 template <int LMAX, bool DIFF>

@@ -328,9 +328,10 @@ th_status solver_cheb_coeffs(thermal_grid* g, double dt, const thermal_solve_opt
 
 // ------------------------------------------------------------------ plan setup
 
-// apply_only: the plan of one preconditioner application (nothing else of it is launched)
+// on_chip: the on-chip inner solve may be taken; apply_only: the plan of one preconditioner
+// application (nothing else of it is launched)
 static th_status make_plan(thermal_grid* g, double dt, const thermal_solve_opts* o, int pdtype, bool transient,
-                           Plan& P, cudaStream_t s, bool apply_only = false) {
+                           Plan& P, cudaStream_t s, bool on_chip = true, bool apply_only = false) {
   P.g = g;
   P.d = grid_dims(g);
   P.gb = grid_blocks(g);
@@ -365,9 +366,16 @@ static th_status make_plan(thermal_grid* g, double dt, const thermal_solve_opts*
   // table; where nx % 4 != 0 a caller who asks for BF16 coefficients gets them, one step
   // per launch.
   if (P.pc == TH_PC_CHEB && (P.prec == TH_PREC_MIXED_IR || (P.prec == TH_PREC_MIXED_IR_BF16 && P.v4)) && P.scaled &&
-      P.uni && o->cheb_fuse == 0) {
-    P.oc_tile = oc_shape(g->nx, g->ny, g->L, P.k);
-    P.oc = P.oc_tile.rows > 0;
+      P.uni && o->cheb_fuse == 0 && on_chip) {
+    P.oc_tile = oc_shape(g->nx, g->ny, g->L, P.k, device_sms());
+    const int sms = P.oc_tile.rows > 0 ? stream_sms(s) : 0;
+    if (sms > 0 && sms < device_sms()) P.oc_tile = oc_shape(g->nx, g->ny, g->L, P.k, sms);
+    if (P.oc_tile.rows > 0) {
+      const th_status st = oc_prepare(g, s);
+      if (st != TH_OK && st != TH_ENOMEM) return st;
+      P.oc = st == TH_OK;
+      if (!P.oc) th_clear_error();  // no memory for its words: the chunk kernels need none
+    }
   }
   // one application on chip needs none of the z-walk kernels (their chunk is tuned once per
   // grid, by timing: most of a first call on a small grid)
@@ -395,7 +403,6 @@ static th_status make_plan(thermal_grid* g, double dt, const thermal_solve_opts*
     // polynomial of the paper runs one step per launch
     // (per-face grids: FP32 faces, so not the BF16-coefficient precision)
     if (P.oc) {
-      TH_TRY(oc_prepare(g, s));
       P.fused = true;
       P.zfin = 0;
     } else if (P.prec != TH_PREC_FP64 && !P.ad && P.v4 && P.scaled && fuse > 1 && P.k > 1 &&
@@ -575,6 +582,41 @@ static int sm_count() {
 }
 
 int device_sms() { return sm_count(); }
+
+int stream_sms(cudaStream_t s) {
+  struct Api {
+    PFN_cuCtxGetCurrent_v4000 current = nullptr;
+    PFN_cuCtxGetDevResource_v12040 ctx_res = nullptr;
+    PFN_cuStreamGetGreenCtx_v12040 green = nullptr;
+    PFN_cuGreenCtxGetDevResource_v12040 green_res = nullptr;
+    Api() {
+      auto get = [](const char* name, unsigned version) -> void* {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion(name, &f, version, cudaEnableDefault, &q) == cudaSuccess) return f;
+        cudaGetLastError();
+        return nullptr;
+      };
+      current = (PFN_cuCtxGetCurrent_v4000)get("cuCtxGetCurrent", 4000);
+      ctx_res = (PFN_cuCtxGetDevResource_v12040)get("cuCtxGetDevResource", 12040);
+      green = (PFN_cuStreamGetGreenCtx_v12040)get("cuStreamGetGreenCtx", 12040);
+      green_res = (PFN_cuGreenCtxGetDevResource_v12040)get("cuGreenCtxGetDevResource", 12040);
+    }
+  };
+  static const Api api;
+  int n = sm_count();
+  CUdevResource r;
+  CUcontext ctx = nullptr;
+  CUgreenCtx part = nullptr;
+  if (api.current && api.ctx_res && api.current(&ctx) == CUDA_SUCCESS && ctx &&
+      api.ctx_res(ctx, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS)
+    n = std::min(n, (int)r.sm.smCount);
+  const bool own = s != nullptr && s != cudaStreamLegacy && s != cudaStreamPerThread;
+  if (own && api.green && api.green_res && api.green(s, &part) == CUDA_SUCCESS && part &&
+      api.green_res(part, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS)
+    n = std::min(n, (int)r.sm.smCount);
+  return n;
+}
 
 template <int LM, int EY, int ST, bool SC, bool LA, bool FI>
 static th_status tb_launch(const Plan& P, const VecSet<float>& V, cudaStream_t st, const Plan::Chunk& c) {
@@ -1137,12 +1179,14 @@ static th_status enq_step_copy(const Plan& P, cudaStream_t st) {
 
 struct GraphKey {
   int kind, prec, pc, k, scaled, pdtype, lz, extrap, fuse, ad_pairs, expire;
+  int oc_rows, oc_halo;  // the on-chip tile, 0: not on chip
   double dt;
   double lam_min, lam_max;  // a caller's Chebyshev interval (its coefficients are baked in)
   bool operator<(const GraphKey& o) const {
-    return std::tie(kind, prec, pc, k, scaled, pdtype, lz, extrap, fuse, ad_pairs, expire, dt, lam_min, lam_max) <
+    return std::tie(kind, prec, pc, k, scaled, pdtype, lz, extrap, fuse, ad_pairs, expire, oc_rows, oc_halo, dt,
+                    lam_min, lam_max) <
            std::tie(o.kind, o.prec, o.pc, o.k, o.scaled, o.pdtype, o.lz, o.extrap, o.fuse, o.ad_pairs, o.expire,
-                    o.dt, o.lam_min, o.lam_max);
+                    o.oc_rows, o.oc_halo, o.dt, o.lam_min, o.lam_max);
   }
 };
 struct GraphEntry {
@@ -1178,6 +1222,7 @@ static th_status capture_body(cudaGraph_t body, cudaStream_t cs, F&& fill) {
   th_status st = fill(cs);
   cudaGraph_t out = nullptr;
   cudaError_t e = cudaStreamEndCapture(cs, &out);
+  if (e != cudaSuccess) cudaGetLastError();
   if (st != TH_OK) return st;
   if (e != cudaSuccess) return th_fail(TH_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
   return TH_OK;
@@ -1326,7 +1371,9 @@ static th_status build_graph(const Plan& P, int kind, const CtlInit& ci, GraphEn
   cudaGraphExec_t ex = nullptr;
   cudaError_t e = cudaGraphInstantiate(&ex, G, 0);
   if (e != cudaSuccess) {
+    cudaGetLastError();
     cudaGraphDestroy(G);
+    g->oc_refused = P.oc && oc_cannot_launch(e);
     return th_fail(TH_ECUDA, "cudaGraphInstantiate failed: %s", cudaGetErrorString(e));
   }
   out->graph = G;
@@ -1468,11 +1515,36 @@ static void fill_stats(const Plan& P, const Ctl& h, float ms, thermal_solve_stat
   st->stage_switches = h.ad_switches;
 }
 
+// Runs f(true), which may solve on chip, and where the device or the part of it that the
+// stream may use has no room for the cooperative launch f(false), the chunk kernels.  (f
+// writes its results last, so nothing is lost.)
+template <class F>
+static th_status with_or_without_oc(thermal_grid* g, F&& f) {
+  g->oc_refused = false;
+  const th_status st = f(true);
+  if (st == TH_OK || !g->oc_refused) return st;
+  th_clear_error();
+  return f(false);
+}
+
+static th_status drive_once(thermal_grid* g, int kind, double dt, const void* const* maps, int n_maps, int pdtype,
+                            int spm, int n_steps, double* T, const thermal_solve_opts* o, thermal_solve_stats* stats,
+                            cudaStream_t s, bool on_chip);
+
 // kind: KIND_STEADY, KIND_STEP or KIND_RUN.  maps/n_maps: power maps; T: host or device.
 th_status solver_drive(thermal_grid* g, int kind, double dt, const void* const* maps, int n_maps, int pdtype,
                        int spm, int n_steps, double* T, const thermal_solve_opts* o, thermal_solve_stats* stats,
                        cudaStream_t s) {
-  if (!g || !T || !maps) return th_fail(TH_EINVAL, "NULL argument");
+  if (!g) return th_fail(TH_EINVAL, "NULL argument");
+  return with_or_without_oc(g, [&](bool on_chip) {
+    return drive_once(g, kind, dt, maps, n_maps, pdtype, spm, n_steps, T, o, stats, s, on_chip);
+  });
+}
+
+static th_status drive_once(thermal_grid* g, int kind, double dt, const void* const* maps, int n_maps, int pdtype,
+                            int spm, int n_steps, double* T, const thermal_solve_opts* o, thermal_solve_stats* stats,
+                            cudaStream_t s, bool on_chip) {
+  if (!T || !maps) return th_fail(TH_EINVAL, "NULL argument");
   if (pdtype != TH_F32 && pdtype != TH_F64) return th_fail(TH_EINVAL, "power dtype must be TH_F32 or TH_F64");
   TH_TRY(validate_opts(o));
   if (o->lanczos_steps > 500) return th_fail(TH_EINVAL, "lanczos_steps must be <= 500");
@@ -1487,7 +1559,7 @@ th_status solver_drive(thermal_grid* g, int kind, double dt, const void* const* 
   if (!transient && !(g->h > 0.0))
     return th_fail(TH_EINVAL, "a steady solve needs h > 0 (h = 0 leaves G singular)");
   const double toff = (kind == KIND_ADJ) ? 0.0 : g->t_amb;  // the adjoint state has no offset
-  TH_TRY(make_plan(g, transient ? dt : 0.0, o, pdtype, transient, P, s));
+  TH_TRY(make_plan(g, transient ? dt : 0.0, o, pdtype, transient, P, s, on_chip));
   P.extrap = (kind == KIND_RUN && o->guess >= 1);
   // quadratic and cubic extrapolation: the vectorised double-float path only (linear elsewhere)
   P.extrap_order = (o->guess >= 2 && P.v4 && o->precision != TH_PREC_FP64 && !P.ad) ? o->guess : 1;
@@ -1524,7 +1596,8 @@ th_status solver_drive(thermal_grid* g, int kind, double dt, const void* const* 
   TH_CUDA(cudaEventRecord(e0, s));
   if (o->use_graph) {
     const GraphKey key{kind,   P.prec, P.pc, P.k, P.scaled, pdtype, o->lanczos_steps, P.extrap ? P.extrap_order : 0,
-                       o->cheb_fuse, P.ad ? P.ad_pairs : 0, P.expire_test, P.transient ? dt : 0.0,
+                       o->cheb_fuse, P.ad ? P.ad_pairs : 0, P.expire_test, P.oc ? P.oc_tile.rows : 0,
+                       P.oc ? P.oc_tile.halo : 0, P.transient ? dt : 0.0,
                        o->cheb_lam_min, o->cheb_lam_max};
     if (!g->graphs) {
       g->graphs = new GraphCache();
@@ -1546,7 +1619,12 @@ th_status solver_drive(thermal_grid* g, int kind, double dt, const void* const* 
       it = g->graphs->m.find(key);
       TH_CUDA(cudaEventRecord(e0, s));
     }
-    TH_CUDA(cudaGraphLaunch(it->second.exec, s));
+    const cudaError_t e = cudaGraphLaunch(it->second.exec, s);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      g->oc_refused = P.oc && oc_cannot_launch(e);
+      return th_fail(TH_ECUDA, "cudaGraphLaunch failed: %s", cudaGetErrorString(e));
+    }
   } else {
     k_ctl_reset<<<1, 1, 0, s>>>(g->ctl, ci);
     TH_CHECK_LAUNCH();
@@ -1661,21 +1739,15 @@ static th_status precond_finish(thermal_grid* g, cudaStream_t s) {
                            "ran out");
 }
 
-extern "C" th_status thermal_precond_apply(thermal_grid* g, double dt, const thermal_solve_opts* opts, const float* r,
-                                           float* z, void* stream) {
-  ABI_BEGIN
-  th_clear_error();
-  if (!g || !r || !z) return th_fail(TH_EINVAL, "NULL argument");
-  TH_TRY(validate_opts(opts));
-  if (opts->lanczos_steps > 500) return th_fail(TH_EINVAL, "lanczos_steps must be <= 500");
-  cudaStream_t s = (cudaStream_t)stream;
+static th_status precond_once(thermal_grid* g, double dt, const thermal_solve_opts* opts, const float* r, float* z,
+                              cudaStream_t s, bool on_chip) {
   thermal_solve_opts o = *opts;
   o.precision = (opts->precision == TH_PREC_MIXED_IR_BF16) ? TH_PREC_MIXED_IR_BF16 : TH_PREC_MIXED_IR;
   Plan P;
   // read r and write z in place of copies, where kernels of this grid's device can
   const BufRange br = buffer_range(r, g->device), bz = buffer_range(z, g->device);
   const int direct = th_direct_buffers(&br, &bz, sizeof(float) * (size_t)g->n, g->device);
-  TH_TRY(make_plan(g, dt, &o, TH_F32, dt > 0.0, P, s, direct > 0));
+  TH_TRY(make_plan(g, dt, &o, TH_F32, dt > 0.0, P, s, on_chip, direct > 0));
   *(volatile int*)g->wait_lost = 0;
   if (P.oc && direct) {  // one launch from r to z
     TH_TRY(oc_enqueue(P, s, 0, r, z));
@@ -1703,6 +1775,18 @@ extern "C" th_status thermal_precond_apply(thermal_grid* g, double dt, const the
   TH_TRY(enq_precond_tail<float>(P, V, s));
   TH_CUDA(cudaMemcpyAsync(z, z_final(P, V), bytes, cudaMemcpyDeviceToDevice, s));
   return precond_finish(g, s);
+}
+
+extern "C" th_status thermal_precond_apply(thermal_grid* g, double dt, const thermal_solve_opts* opts, const float* r,
+                                           float* z, void* stream) {
+  ABI_BEGIN
+  th_clear_error();
+  if (!g || !r || !z) return th_fail(TH_EINVAL, "NULL argument");
+  TH_TRY(validate_opts(opts));
+  if (opts->lanczos_steps > 500) return th_fail(TH_EINVAL, "lanczos_steps must be <= 500");
+  return with_or_without_oc(g, [&](bool on_chip) {
+    return precond_once(g, dt, opts, r, z, (cudaStream_t)stream, on_chip);
+  });
   ABI_END
 }
 

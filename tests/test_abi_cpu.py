@@ -198,3 +198,24 @@ def test_dynamic_shared_memory_states_its_alignment():
                 m = re.search(r"__align__\((\d+)\)", quals)
                 assert m and int(m.group(1)) >= 16, (os.path.basename(f), name)
     assert cast > 0
+
+
+def test_on_chip_tiles_fit_the_sms(lib):
+    """The on-chip tile is chosen for the SMs a launch may use: one tile each, and none where
+    they do not fit."""
+    class Shape(C.Structure):
+        _fields_ = [("rows", C.c_int), ("halo", C.c_int)]
+
+    f = lib._Z8oc_shapeiiiii
+    f.restype = Shape
+    for nx, ny, L, k in ((64, 64, 4, 30), (200, 160, 8, 12), (301, 203, 8, 30), (130, 70, 4, 12), (24, 8, 5, 5),
+                         (76, 37, 10, 8), (288, 288, 8, 10), (1, 1, 12, 2)):
+        for sms in (1, 8, 16, 72, 132, 152):
+            t = f(nx, ny, L, k, sms)
+            if t.rows:
+                tx, ty = 32 - 2 * t.halo, t.rows - 2 * t.halo
+                assert tx >= t.halo and ty >= t.halo >= 2 and -(-nx // tx) * -(-ny // ty) <= sms
+            else:  # the largest tile of the capacity does not fit either
+                rows = 24 if L > 8 else 32
+                assert -(-nx // 28) * -(-ny // (rows - 4)) > sms
+    assert f(64, 64, 4, 30, 152).rows and not f(64, 64, 4, 30, 2).rows
