@@ -177,6 +177,8 @@ th_status grid_ensure_dg64(thermal_grid* g, double dt, cudaStream_t s);
 struct MGHier;
 void mg_free(MGHier* h);
 th_status grid_ensure_mg(thermal_grid* g, double dt, cudaStream_t s);
+// the cycles that follow run on s (or in a graph launched there); false: it has part of the SMs
+bool mg_set_stream(thermal_grid* g, cudaStream_t s);
 th_status mg_vcycle(thermal_grid* g, const float* r, float* z, cudaStream_t s);
 // The multigrid hierarchy of one grid as plain device pointers, for the batched
 // persistent solve: per level the dimensions, the per-cell coefficients and Thomas

@@ -123,7 +123,9 @@ __global__ void k_mg_zfactors(int nx, int ny, int L, const float* __restrict__ g
 // 60.4 / 60.7 / 131.9 / 181.3, at 6 blocks 62.3 / 74.9 / 131.1 / 183.6.
 constexpr int MG_EY = 8;
 constexpr unsigned MG_MINB = 4;
-constexpr int MG_CLUSTER = 16;  // blocks of the cluster (8 where 16 cannot be scheduled)
+// blocks of the cluster (8 where 16 cannot be scheduled; 1 on a stream that has only part of
+// the SMs, whose clusters may be smaller: slow, but any SM takes it)
+constexpr int MG_CLUSTER = 16;
 
 template <int LMAX>
 struct MGCLev {
@@ -405,6 +407,7 @@ struct MGHier {
   double dt = -1.0;
   std::vector<MGLevelH> lv;
   int cluster = 0;    // blocks of k_mg_levels' cluster (0: not looked up yet)
+  bool whole = true;  // the current call's stream has all SMs
   bool uni = false;   // finest level from the layer table
   MGUni<32> tab{};    // its coefficients and Thomas factors (first L layers used)
   // Levels whose coefficients depend only on the layer (and on which in-plane
@@ -608,6 +611,11 @@ th_status grid_ensure_mg(thermal_grid* g, double dt, cudaStream_t s) {
   return TH_OK;
 }
 
+bool mg_set_stream(thermal_grid* g, cudaStream_t s) {
+  g->mg->whole = stream_sms(s) >= device_sms();
+  return g->mg->whole;
+}
+
 // the table of level k (layer-uniform levels only)
 template <int LMAX>
 static MGUni<LMAX> uni_of(const MGHier* h, int k) {
@@ -692,7 +700,7 @@ static th_status mg_levels(thermal_grid* g, int k0, const float* b0, float* z, c
     if (cudaOccupancyMaxActiveClusters(&fits, kern, &c) != cudaSuccess) cudaGetLastError();
     h->cluster = fits > 0 ? MG_CLUSTER : 8;
   }
-  blocks(h->cluster);
+  blocks(h->whole ? h->cluster : 1);
   TH_CUDA(cudaLaunchKernelEx(&c, kern, g->ctl, (const MGCLev<LMAX>*)h->dlv, g->L, k0, nl, h->nc, (const float*)h->cinv,
                              b0, z, g->partials, g->partials_stride, g->counters));
   return TH_OK;

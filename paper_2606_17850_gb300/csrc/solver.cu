@@ -57,6 +57,7 @@ struct Plan {
   bool stream = false;  // the chunks run as register streams (kernels_stream.cuh), not tiles
   bool oc = false;     // inner PCG on chip (pcg_oc.cu)
   OCShape oc_tile{0, 0};
+  bool mg_part = false;  // multigrid on a stream with part of the SMs
   int tb_lmax = 8;  // layer capacity of the fused kernel (8: 32 x 32 tiles, 12: 32 x 24)
   std::vector<Chunk> chunks;
   int zfin = -1;  // pool index of the preconditioned vector (-1: the per-step rule)
@@ -357,7 +358,10 @@ static th_status make_plan(thermal_grid* g, double dt, const thermal_solve_opts*
     P.ad_pairs = std::max(1, (chk + 1) / 2);
   }
   if (P.pc == TH_PC_ZLINE) TH_TRY(grid_ensure_zline(g, dt, s));
-  if (P.pc == TH_PC_MG) TH_TRY(grid_ensure_mg(g, dt, s));
+  if (P.pc == TH_PC_MG) {
+    TH_TRY(grid_ensure_mg(g, dt, s));
+    P.mg_part = !mg_set_stream(g, s);
+  }
   if (P.prec == TH_PREC_FP64) TH_TRY(grid_ensure_dg64(g, dt, s));
   P.v4 = (g->nx % 4 == 0);
   P.uni = g->uniform;
@@ -1180,13 +1184,14 @@ static th_status enq_step_copy(const Plan& P, cudaStream_t st) {
 struct GraphKey {
   int kind, prec, pc, k, scaled, pdtype, lz, extrap, fuse, ad_pairs, expire;
   int oc_rows, oc_halo;  // the on-chip tile, 0: not on chip
+  int mg_part;
   double dt;
   double lam_min, lam_max;  // a caller's Chebyshev interval (its coefficients are baked in)
   bool operator<(const GraphKey& o) const {
-    return std::tie(kind, prec, pc, k, scaled, pdtype, lz, extrap, fuse, ad_pairs, expire, oc_rows, oc_halo, dt,
-                    lam_min, lam_max) <
+    return std::tie(kind, prec, pc, k, scaled, pdtype, lz, extrap, fuse, ad_pairs, expire, oc_rows, oc_halo,
+                    mg_part, dt, lam_min, lam_max) <
            std::tie(o.kind, o.prec, o.pc, o.k, o.scaled, o.pdtype, o.lz, o.extrap, o.fuse, o.ad_pairs, o.expire,
-                    o.oc_rows, o.oc_halo, o.dt, o.lam_min, o.lam_max);
+                    o.oc_rows, o.oc_halo, o.mg_part, o.dt, o.lam_min, o.lam_max);
   }
 };
 struct GraphEntry {
@@ -1597,7 +1602,7 @@ static th_status drive_once(thermal_grid* g, int kind, double dt, const void* co
   if (o->use_graph) {
     const GraphKey key{kind,   P.prec, P.pc, P.k, P.scaled, pdtype, o->lanczos_steps, P.extrap ? P.extrap_order : 0,
                        o->cheb_fuse, P.ad ? P.ad_pairs : 0, P.expire_test, P.oc ? P.oc_tile.rows : 0,
-                       P.oc ? P.oc_tile.halo : 0, P.transient ? dt : 0.0,
+                       P.oc ? P.oc_tile.halo : 0, P.mg_part, P.transient ? dt : 0.0,
                        o->cheb_lam_min, o->cheb_lam_max};
     if (!g->graphs) {
       g->graphs = new GraphCache();

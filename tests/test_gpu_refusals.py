@@ -197,17 +197,47 @@ def test_refused_cooperative_launch_takes_the_chunks(faked, nx, ny, mk, k):
     g.close()
 
 
+def _part_stream(faked):
+    ptr, got = C.c_void_p(), C.c_uint()
+    if faked.green_stream(16, C.byref(ptr), C.byref(got)) != 0:
+        pytest.skip("no green contexts here")
+    return ptr, got.value
+
+
+@pytest.mark.parametrize("nx,ny,mk", [(64, 40, "c1"), (200, 150, "c2"), (131, 77, "mol")])
+def test_vcycle_on_part_of_the_device(faked, nx, ny, mk):
+    """The V-cycle on a stream with 16 SMs, where a cluster of 16 blocks may have no place:
+    the same vector, and the solves' results."""
+    from paper_2606_17850_gb300 import ThermalGrid
+    ptr, _ = _part_stream(faked)
+    st = STACKS[mk]()
+    P, r = _power(st, nx, ny), torch.from_numpy(ti.random_vector(nx * ny * st.L, 5).astype(np.float32)).cuda()
+    g = ThermalGrid.from_stack(nx, ny, st)
+
+    def calls():
+        T = [g.solve_steady(P, precond="mg", tol_rel=1e-9, use_graph=q)[0] - st.t_amb for q in (0, 1)]
+        return [g.precond(r, 0.0, precond="mg")] + T
+
+    want = calls()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.ExternalStream(ptr.value)):
+        have = calls()
+        torch.cuda.synchronize()
+    assert torch.equal(have[0], want[0])
+    for x, y in zip(have[1:], want[1:]):
+        assert (x - y).abs().max().item() <= 1e-6 * y.abs().max().item()
+    g.close()
+
+
 def test_on_chip_tiles_fit_the_streams_part_of_the_device(faked):
     """A stream of a green context with 16 SMs: grids with more tiles run the chunk kernels,
     smaller ones stay on chip."""
     from paper_2606_17850_gb300 import ThermalGrid
-    ptr, got = C.c_void_p(), C.c_uint()
-    if faked.green_stream(16, C.byref(ptr), C.byref(got)) != 0:
-        pytest.skip("no green contexts here")
+    ptr, got = _part_stream(faked)
     sms = faked._Z10stream_smsP11CUstream_st
     sms.argtypes = [C.c_void_p]
     whole = torch.cuda.get_device_properties(0).multi_processor_count
-    assert sms(ptr) == got.value < whole and sms(None) == whole
+    assert sms(ptr) == got < whole and sms(None) == whole
     part = torch.cuda.ExternalStream(ptr.value)
     for nx, ny, mk, k, fits in ((200, 160, "c2", 12, 0), (288, 201, "c1", 9, 0), (24, 8, "c2", 9, 1), (60, 41, "c1", 12, 1)):
         st = STACKS[mk]()
