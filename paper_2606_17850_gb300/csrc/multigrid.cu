@@ -399,7 +399,8 @@ struct MGLevelH {
   long long n = 0;
   const float *gx = nullptr, *gy = nullptr, *gz = nullptr;  // level 0: the grid's FP32 faces
   float *own_gx = nullptr, *own_gy = nullptr, *own_gz = nullptr;
-  float *s = nullptr, *m = nullptr, *w = nullptr;
+  float *s = nullptr;
+  float *m = nullptr, *w = nullptr;  // Thomas factors, from the first time the level is not layer-uniform
   float *x = nullptr, *xt = nullptr, *b = nullptr;
 };
 
@@ -408,8 +409,6 @@ struct MGHier {
   std::vector<MGLevelH> lv;
   int cluster = 0;    // blocks of k_mg_levels' cluster (0: not looked up yet)
   bool whole = true;  // the current call's stream has all SMs
-  bool uni = false;   // finest level from the layer table
-  MGUni<32> tab{};    // its coefficients and Thomas factors (first L layers used)
   // Levels whose coefficients depend only on the layer (and on which in-plane
   // neighbours exist): the finest level of a layer-uniform grid and every coarser
   // level reached through complete 2 x 2 aggregates (even nx, ny above it).  Their
@@ -480,8 +479,6 @@ th_status grid_ensure_mg(thermal_grid* g, double dt, cudaStream_t s) {
     for (size_t k = 0; k < h->lv.size(); ++k) {
       MGLevelH& l = h->lv[k];
       TH_TRY(mg_alloc(&l.s, l.n));
-      TH_TRY(mg_alloc(&l.m, l.n));
-      TH_TRY(mg_alloc(&l.w, l.n));
       TH_TRY(mg_alloc(&l.xt, l.n));
       if (k == 0) {
         l.gx = g->f32.gx;
@@ -513,7 +510,6 @@ th_status grid_ensure_mg(thermal_grid* g, double dt, cudaStream_t s) {
     TH_CHECK_LAUNCH();
   }
   // layer-uniform levels: coefficients and Thomas factors per in-plane case
-  h->uni = g->uniform;
   const size_t nlv = h->lv.size();
   h->luni.assign(nlv, 0);
   h->ltab.assign(nlv, MGUni<32>{});
@@ -537,7 +533,7 @@ th_status grid_ensure_mg(thermal_grid* g, double dt, cudaStream_t s) {
         }
       }
   };
-  if (h->uni) {
+  if (g->uniform) {
     const LayerTab& T = g->tab_host;
     MGUni<32>& t0 = h->ltab[0];
     std::memset(&t0, 0, sizeof(t0));
@@ -571,11 +567,12 @@ th_status grid_ensure_mg(thermal_grid* g, double dt, cudaStream_t s) {
       factors(t);
       h->luni[k + 1] = 1;
     }
-    h->tab = h->ltab[0];
   }
   for (size_t k = 0; k < nlv; ++k) {  // a layer-uniform level's factors are in its table
-    const MGLevelH& l = h->lv[k];
+    MGLevelH& l = h->lv[k];
     if (h->luni[k]) continue;
+    if (!l.m) TH_TRY(mg_alloc(&l.m, l.n));
+    if (!l.w) TH_TRY(mg_alloc(&l.w, l.n));
     k_mg_zfactors<<<col_grid(l.nx, l.ny), dim3(32, 8), 0, s>>>(l.nx, l.ny, L, l.gx, l.gy, l.gz, l.s, l.m, l.w);
     TH_CHECK_LAUNCH();
   }

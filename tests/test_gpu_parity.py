@@ -1239,3 +1239,35 @@ def test_bf16_coefficients_read_where_nx_is_ragged(nx, ny, mk, k):
         assert torch.equal(z, g.precond(r, dt, precision="mixed_bf16", precond="cheb", cheb_degree=k, cheb_fuse=1))
         z32 = g.precond(r, dt, precision="mixed", precond="cheb", cheb_degree=k)
         assert (z - z32).abs().max().item() > 1e-5 * z32.abs().max().item()
+
+
+def test_mg_memory_and_a_map_later():
+    """A layer-table grid's hierarchy holds no per-cell Thomas factors (sizes of its arrays
+    and a tenth for the allocator's granules); a conductivity map later, and the table
+    again, give the V-cycles of grids that began so."""
+    nx, ny, st = 1024, 768, ti.stack_c2()
+    n = nx * ny * st.L
+    r = cuda(ti.random_vector(n, 5).astype(np.float32))
+    g = grid_of(nx, ny, st)
+    g.precond(r, 0.0, precond="jacobi")
+    g2 = grid_of(64, 48, st)
+    g2.precond(r[:g2.n], 0.0, precond="mg")  # the kernels are loaded
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    z0 = torch.empty_like(r)
+    z0.copy_(g.precond(r, 0.0, precond="mg"))
+    torch.cuda.synchronize()
+    held = free0 - torch.cuda.mem_get_info()[0]
+    # finest s, xt; coarse gx, gy, gz, s, xt, x, b; z0 and the result from torch
+    want = 4 * n * (2 + 7 / 3) + 4 * (64 * st.L) ** 2
+    assert held <= 1.1 * want + 2 * 4 * n, (held, want)
+    for kmap in (1, 0):
+        kc = _kmap(st, nx, ny, 21)
+        h = grid_of(nx, ny, st)
+        if kmap:
+            g.set_conductivity_map(cuda(kc))
+            h.set_conductivity_map(cuda(kc))
+        else:
+            g.set_conductivity(list(st.k()))
+        assert torch.equal(g.precond(r, 0.0, precond="mg"), h.precond(r, 0.0, precond="mg"))
+    assert torch.equal(g.precond(r, 0.0, precond="mg"), z0)
