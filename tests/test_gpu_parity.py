@@ -1271,3 +1271,61 @@ def test_mg_memory_and_a_map_later():
             g.set_conductivity(list(st.k()))
         assert torch.equal(g.precond(r, 0.0, precond="mg"), h.precond(r, 0.0, precond="mg"))
     assert torch.equal(g.precond(r, 0.0, precond="mg"), z0)
+
+
+def test_handles_on_threads_and_streams():
+    """Two handles at a time, each on a thread and a stream of its own: on chip (tiles for
+    nearly every SM, so that the two take turns), streams, tiles and V-cycles give what they
+    give alone.  The threads of a fresh process meet at its first use of each kernel."""
+    import subprocess
+    import sys
+    from conftest import ROOT
+    src = """
+import threading, sys
+sys.path.insert(0, '.')
+import numpy as np, torch
+import thermal_inputs as ti
+import __graft_entry__ as ge
+ge.build()
+from paper_2606_17850_gb300 import ThermalGrid
+st = ti.stack_c2()
+jobs = [(280, 281, dict(precond='cheb', cheb_degree=12)), (280, 280, dict(precond='cheb', cheb_degree=9)),
+        (772, 771, dict(precond='cheb', cheb_degree=9)), (520, 200, dict(precond='cheb', cheb_degree=9, cheb_fuse=3)),
+        (200, 150, dict(precond='mg'))]
+def work(which, out, start):
+    try:
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            start.wait()
+            for i in which:
+                nx, ny, o = jobs[i]
+                g = ThermalGrid.from_stack(nx, ny, st)
+                rng = np.random.default_rng(i)
+                r = torch.from_numpy(rng.standard_normal(g.n, dtype=np.float32)).cuda()
+                P = torch.from_numpy(rng.random(g.n, dtype=np.float32) * np.float32(1e-4)).cuda()
+                z = [g.precond(r, 1e-4, **o) for _ in range(20)]
+                T = [g.solve_steady(P, tol_rel=1e-7, use_graph=q, **o)[0] for q in (0, 1)]
+                s.synchronize()
+                assert all(torch.equal(z[0], v) for v in z)
+                out[i] = (z[0].cpu(), [t.cpu() for t in T])
+    except BaseException as e:
+        out['error'] = e
+        raise
+def both(a, b):
+    outs, start = [{}, {}], threading.Barrier(2)
+    th = [threading.Thread(target=work, args=(w, o, start)) for w, o in zip((a, b), outs)]
+    [t.start() for t in th]; [t.join() for t in th]
+    assert not any('error' in o for o in outs), outs
+    return outs
+first = both([2, 0, 1, 3, 4], [2, 1, 0, 4, 3])
+alone = {}
+work(range(len(jobs)), alone, threading.Barrier(1))
+for o in first + both([0, 0, 1], [1, 0, 0]):
+    for i, (z, T) in o.items():
+        assert torch.equal(z, alone[i][0]), i
+        for x, y in zip(T, alone[i][1]):
+            assert (x - y).abs().max() <= 1e-5 * (y - st.t_amb).abs().max(), i
+print('same')
+"""
+    r = subprocess.run([sys.executable, "-c", src], capture_output=True, text=True, cwd=ROOT, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip().endswith("same"), r.stdout + r.stderr
