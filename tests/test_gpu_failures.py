@@ -153,3 +153,59 @@ def test_precond_wait_expiry_reported(nx, ny, mk, kmap, fuse, inplace):
     assert torch.equal(apply(), z0)
     r0[5] = float("nan")
     apply()                    # not an error of the application
+
+
+@pytest.mark.parametrize("graph", [0, 1])
+@pytest.mark.parametrize("kind", ["steady", "run"])
+def test_streaming_wait_expiry_reported(graph, kind):
+    """The bounded wait of the streaming chunks, in solves: TH_ECUDA, and the next solve on
+    the grid is the one before."""
+    from paper_2606_17850_gb300 import ThermalError
+    st = ti.stack_c1()
+    nx, ny, dt = 448, 451, 1e-4
+    g = _grid(nx, ny, st)
+    P = torch.from_numpy(ti.power_cells(st, nx, ny, [ti.density_uniform_hotspots(nx, ny, 4)
+                                                     for _ in st.power_layers()], np.float32)).cuda()
+    opts = dict(precision="mixed", precond="cheb", cheb_degree=12, tol_rel=1e-9, use_graph=graph)
+
+    def solve(**kw):
+        if kind == "steady":
+            return g.solve_steady(P, **opts, **kw)[0]
+        T = torch.full((g.n,), st.t_amb, dtype=torch.float64, device="cuda")
+        g.run_transient([P], 2, 3, dt, T, **opts, **kw)
+        return T
+
+    ref = solve()
+    with pytest.raises(ThermalError) as e:
+        solve(test_wait_expire=1)
+    assert e.value.status == 3 and "timed out" in str(e.value)
+    torch.cuda.synchronize()   # the context is still usable
+    assert (solve() - ref).abs().max().item() <= 1e-6 * (ref - st.t_amb).abs().max().item()
+
+
+@pytest.mark.parametrize("graph", [0, 1])
+@pytest.mark.parametrize("nx", [36, 37])
+@pytest.mark.parametrize("lam,k,status", [((0.05, 1.6), 20, 5), ((0.05, 0.9), 40, 6)])
+def test_breakdown_on_chip(nx, lam, k, status, graph):
+    """A caller's interval whose upper end lies below the checkerboard mode's eigenvalue
+    makes the scaled polynomial of even degree negative there: r^T z < 0 is TH_EBREAKDOWN;
+    where z is so large that its products overflow FP32 it is TH_ENONFINITE, as one step
+    per launch reports.  The oracle confirms both on the host."""
+    from paper_2606_17850_gb300 import ThermalError
+    st = ti.stack_c2()
+    ny = 29
+    A = disc.assemble(nx, ny, st)
+    D = A.diagonal()
+    P = _checkerboard(nx, ny, st.L)
+    z = krylov.chebyshev(lambda v: (A @ v) / D, P / D, *lam, k)
+    r = P / np.linalg.norm(P)
+    zn = z / np.linalg.norm(P)
+    assert r @ zn < 0
+    assert ((zn * (A @ zn)).max() > 1e40) == (status == 6) and ((zn * (A @ zn)).max() < 1e30) == (status == 5)
+    g = _grid(nx, ny, st)
+    for fuse in (0, 1):
+        with pytest.raises(ThermalError) as e:
+            g.solve_steady(torch.from_numpy(P).cuda(), precision="mixed", precond="cheb", cheb_degree=k, cheb_fuse=fuse,
+                           cheb_lam_min=lam[0], cheb_lam_max=lam[1], tol_rel=1e-10, use_graph=graph)
+        assert e.value.status == status, fuse
+    _normal_solve_matches_oracle(g, nx, ny, st, precision="mixed", cheb_degree=8, use_graph=graph)

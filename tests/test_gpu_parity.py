@@ -1329,3 +1329,16 @@ print('same')
 """
     r = subprocess.run([sys.executable, "-c", src], capture_output=True, text=True, cwd=ROOT, timeout=300)
     assert r.returncode == 0 and r.stdout.strip().endswith("same"), r.stdout + r.stderr
+
+
+def test_streaming_sizes_are_streamed():
+    """The sizes that the streaming tests list take the streaming form on this device (the
+    choice is a cost model of its SMs), and those of the tile tests do not."""
+    import ctypes as C
+    from paper_2606_17850_gb300 import _lib
+    pays = _lib.load()._Z16cheb_stream_paysiii
+    pays.restype = C.c_bool
+    for nx, ny, mk in ((772, 771, "c2"), (1024, 1024, "c2"), (2052, 263, "c2"), (260, 2051, "l7"), (448, 451, "c1"),
+                       (1028, 520, "l6"), (1084, 700, "l5"), (772, 768, "c2")):
+        assert pays(nx, ny, STACKS[mk]().L), (nx, ny, mk)
+    assert not pays(76, 37, 8) and not pays(128, 128, 4) and not pays(1024, 1024, 10) and not pays(1023, 1024, 8)
