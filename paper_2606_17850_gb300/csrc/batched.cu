@@ -328,13 +328,13 @@ __device__ void mg_phase(const BArgs& A, int k, MGUni<8>& tab, F body) {
   for (int t = t0 + (int)blockIdx.x; t < t1; t += gridDim.x) {
     const int2 e = __ldg(A.mgt + t);
     if (e.x != cur) {
-      __syncthreads();
       __syncthreads();  // nobody is in the tile before
       if (tid == 0) s_act = active(A.inst[e.x].ctl, ACT_INNER);
       const MGBLevel& l = A.mg[e.x].lv[k];
       if (l.uni) {  // the level's table into shared memory
         const int* src = reinterpret_cast<const int*>(&l.t);
-        for (int i = tid; i < (int)(sizeof(MGUni<8>) / 4); i += block_threads()) reinterpret_cast<int*>(&tab)[i] = __ldg(src + i);
+        for (int i = tid; i < (int)(sizeof(MGUni<8>) / 4); i += block_threads())
+          reinterpret_cast<int*>(&tab)[i] = __ldg(src + i);
       }
       cur = e.x;
     }
@@ -401,8 +401,9 @@ __device__ void mg_vcycle_batched(const BArgs& A, cg::grid_group& grid) {
       float* out = (k == 0) ? I.zc[0] : l.xt;
       const MGDev v = mg_dev(D, k, I.d.L);
       float rz;
-      if (l.uni) rz = mgt_up<8, true, TH_BY4, false, true>(v, tab, tile % tbx, tile / tbx, b, xin, xc, c.nx, c.ny, out, xs);
-      else rz = mgt_up<8, false, TH_BY4, false, true>(v, c_mg_none, tile % tbx, tile / tbx, b, xin, xc, c.nx, c.ny, out, xs);
+      const int tx = tile % tbx, ty = tile / tbx;
+      if (l.uni) rz = mgt_up<8, true, TH_BY4, false, true>(v, tab, tx, ty, b, xin, xc, c.nx, c.ny, out, xs);
+      else rz = mgt_up<8, false, TH_BY4, false, true>(v, c_mg_none, tx, ty, b, xin, xc, c.nx, c.ny, out, xs);
       if (k == 0) {  // r^T z of the tile
         const float ws = warp_sum(rz);
         if ((tid & 31) == 0) red[tid >> 5] = (double)ws;

@@ -147,8 +147,8 @@ __global__ void __launch_bounds__(32, LMAX <= 4 ? 14 : (LMAX <= 6 ? 10 : 8))
   unsigned off = 4u * (unsigned)(gx + nx * (y0 - 2 * S));  // bytes to the cell of the row that step S forms, in its layer
 
   // one row: GEN handles rows at and outside the y edges and the strip's first rows
-  auto row = [&](auto rot, auto gen) {
-    constexpr int O = decltype(rot)::v % 3, M = (O + 1) % 3, N = (O + 2) % 3;
+  auto row = [&](auto gen) {
+    constexpr int O = 0, M = 1, N = 2;  // older, middle and new row of a level
     constexpr bool GEN = decltype(gen)::v != 0;
     const int t = y0 - S + it;
     __syncwarp();  // every lane is done with the ring slots that the next fetch reuses
@@ -257,8 +257,8 @@ __global__ void __launch_bounds__(32, LMAX <= 4 ? 14 : (LMAX <= 6 ? 10 : 8))
   if (ok && !done) {
 #pragma unroll 1
     while (it < nit && ok) {
-      if (it >= lo && it < hi) row(StInt<0>{}, StInt<0>{});
-      else row(StInt<0>{}, StInt<1>{});
+      if (it >= lo && it < hi) row(StInt<0>{});
+      else row(StInt<1>{});
       shift();
     }
   }

@@ -11,7 +11,10 @@
 // the running kernel (loads that bypass L1).
 //
 // Order of a cell's product: s x, then the x, y and z faces (+ before -); an aggregate is
-// summed x pairs first.
+// summed x pairs first: the operations of the kernels that read every neighbour from global
+// memory, in their order.  A V-cycle's error against 64 bits over 24 right-hand sides on four
+// grids (5e-8 to 1.2e-7 of ||z||) is 0.53 to 1.43 of theirs, 0.94 in the mean: which way FP32
+// rounds, not how much.
 #pragma once
 
 #include "mg_device.cuh"

@@ -110,9 +110,9 @@ __global__ void k_mg_zfactors(int nx, int ny, int L, const float* __restrict__ g
 // with more tiles than a cluster has blocks run them as launches of their own; the levels
 // below run, way down, coarsest solve and way up, in one launch of a single cluster whose
 // blocks meet at its hardware barrier: they are bound by the latency of a pass, not by
-// work, and a grid has four or five of them.  Measured V-cycles with r^T z, before (two
-// launches down and one up per level, r^T z apart) and now: 64^2 x 4 42 -> 18.5 us, 128^2 x
-// 8 69 -> 31, 357 x 301 x 8 168 -> 61, 512^2 x 8 126 -> 60, 1024^2 x 8 225 -> 132, 1024^2 x
+// work, and a grid has two or three of them.  Measured V-cycles with r^T z, before (two
+// launches down and one up per level, r^T z apart) and now: 64^2 x 4 42 -> 18.8 us, 128^2 x
+// 8 69 -> 29, 357 x 301 x 8 168 -> 61, 512^2 x 8 126 -> 60, 1024^2 x 8 225 -> 126, 1024^2 x
 // 10 287 -> 181.  (All these levels in one cooperative grid with a barrier in memory: 84 ->
 // 108 us at 512^2; a phase there costs 5 us.)  The finest level is bound by the latency of
 // a tile's load - solve - store chain at 32 warps an SM (2.3 to 2.5 TB/s).
@@ -712,16 +712,16 @@ static th_status mg_half(thermal_grid* g, int k, bool up, const float* b, float*
   const MGUni<LMAX> U = uni_of<LMAX>(h, k);
   const dim3 gr((l.nx + MGT_EX - 3) / (MGT_EX - 2), (l.ny + MG_EY - 3) / (MG_EY - 2)), bl(MGT_EX, MG_EY);
   constexpr size_t sm = mg_xs_bytes<LMAX>();
+  static_assert(sm <= (40u << 10), "a tile needs the opt-in for larger shared memory");
   auto launch = [&](auto* kern, dim3 blocks, auto... a) -> th_status {
-    if (sm > (40u << 10)) TH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     th_launch(kern, blocks, bl, sm, s, a...);
     TH_CHECK_LAUNCH();
     return TH_OK;
   };
   if (!up) return launch(k_mg_down<LMAX, UNI>, gr, g->ctl, dev_of(l, g->L), U, b, x, c.nx, c.ny, c.b);
   if (k == 0)
-    return launch(k_mg_up<LMAX, UNI, true>, std::min(gr.x * gr.y, (LMAX <= 12 ? MG_MINB : 1u) * device_sms()), g->ctl, dev_of(l, g->L), U, b, x, xc, c.nx, c.ny, z, g->partials,
-                  g->partials_stride, g->counters);
+    return launch(k_mg_up<LMAX, UNI, true>, std::min(gr.x * gr.y, (LMAX <= 12 ? MG_MINB : 1u) * device_sms()), g->ctl,
+                  dev_of(l, g->L), U, b, x, xc, c.nx, c.ny, z, g->partials, g->partials_stride, g->counters);
   return launch(k_mg_up<LMAX, UNI, false>, gr, g->ctl, dev_of(l, g->L), U, b, x, xc, c.nx, c.ny, z, g->partials,
                 g->partials_stride, g->counters);
 }
@@ -739,8 +739,10 @@ static th_status mg_cycle(thermal_grid* g, const float* r, float* z, cudaStream_
     return mg_uni(h, k) ? mg_half<LMAX, true>(g, k, up, b, x, xc, out, s)
                         : mg_half<LMAX, false>(g, k, up, b, x, xc, out, s);
   };
-  // first level of the cluster's: two tiles a block (one: 64^2 x 4 22.5 instead of 20.5 us;
-  // eight: 512^2 x 8 78 instead of 66 us)
+  // first level of the cluster's: at most two tiles a block (so a 64 x 64 level, of 33 tiles,
+  // is not).  V-cycles (us) at two / three / four / eight: 64^2 x 4 18.8 / 20.5 / 20.5 / 20.5,
+  // 200 x 150 x 8 38.9 / 38.9 / 45.1 / 45.1, 512^2 x 8 60.1 / 63.2 / 63.3 / 77.9, 1024^2 x 10
+  // 180.7 / 186.4 / 186.5 / 205.3
   int k0 = 0;
   while (k0 < nl - 1 && mgt_tiles<MG_EY>(h->lv[k0].nx, h->lv[k0].ny) > 2 * MG_CLUSTER) ++k0;
   for (int k = 0; k < k0; ++k) TH_TRY(half(k, false));

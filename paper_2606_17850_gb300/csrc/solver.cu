@@ -258,9 +258,9 @@ static th_status tune_zchunk(thermal_grid* g, cudaStream_t s) {
     if (ci > 0 && zc == cands[ci - 1]) continue;
     const dim3 gb = v4_blocks(g, zc);
     auto run = [&]() {
-      TH_UNI(g->uniform, th_launch(k_cheb_v4<float, true, false, U>, gb, dim3(TH_BX, TH_BY4), 0, s, 
-                             d, zc, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz, g->tab, g->r32, g->zc32[0],
-                             g->zc32[1], g->zc32[2], 0.5f, 0.5f, g->partials, g->partials_stride, g->counters));
+      TH_UNI(g->uniform, th_launch(k_cheb_v4<float, true, false, U>, gb, dim3(TH_BX, TH_BY4), 0, s, d, zc, g->ctl,
+                                   g->f32.gx, g->f32.gy, g->f32.gz, g->tab, g->r32, g->zc32[0], g->zc32[1],
+                                   g->zc32[2], 0.5f, 0.5f, g->partials, g->partials_stride, g->counters));
     };
     run();
     TH_CUDA(cudaEventRecord(e0, s));
@@ -500,9 +500,9 @@ static th_status enq_update(const Plan& P, const VecSet<TV>& V, cudaStream_t st,
     if (P.v4) {
 #define TH_UPD4(ZM)                                                                                        \
   TH_UNI(P.uni && P.d.n < (1LL << 33),                                                                     \
-         th_launch(k_update_v4<INIT, ZM, U>, P.nbr4, 256, 0, st, P.d.n / 4, ctl, xw, pp, V.r, V.mu, V.invd, V.zc[0], \
-                                                          zs, P.scaled, rz1, scale_r, g->partials,          \
-                                                          g->partials_stride, g->counters, P.d, g->tab))
+         th_launch(k_update_v4<INIT, ZM, U>, P.nbr4, 256, 0, st, P.d.n / 4, ctl, xw, pp, V.r, V.mu, V.invd,  \
+                   V.zc[0], zs, P.scaled, rz1, scale_r, g->partials, g->partials_stride, g->counters, P.d,   \
+                   g->tab))
       switch (P.pc) {
         case TH_PC_NONE: TH_UPD4(0); break;
         case TH_PC_JACOBI: TH_UPD4(1); break;
@@ -518,8 +518,8 @@ static th_status enq_update(const Plan& P, const VecSet<TV>& V, cudaStream_t st,
     }
   }
 #define TH_UPD(ZM)                                                                                          \
-  th_launch(k_update<TV, INIT, ZM>, P.gb, P.tb, 0, st, P.d, ctl, xw, pp, V.r, V.mu, V.invd, V.zc[0], zs, P.scaled, \
-                                                rz1, scale_r, g->partials, g->partials_stride, g->counters)
+  th_launch(k_update<TV, INIT, ZM>, P.gb, P.tb, 0, st, P.d, ctl, xw, pp, V.r, V.mu, V.invd, V.zc[0], zs,     \
+            P.scaled, rz1, scale_r, g->partials, g->partials_stride, g->counters)
   switch (P.pc) {
     case TH_PC_NONE: TH_UPD(0); break;
     case TH_PC_JACOBI: TH_UPD(1); break;
@@ -669,9 +669,9 @@ static th_status tb_launch(const Plan& P, const VecSet<float>& V, cudaStream_t s
                                (int)smem));
   const int nblk = std::min(ntiles, sm_count());
   if (nblk > g->partials_stride) return th_fail(TH_ESTATE, "partials buffer smaller than the temporal-blocking grid");
-  th_launch(k_cheb_tb<LM, EY, ST, SC, LA, FI>, nblk, dim3(TB_EX, EY), smem, st, 
-      P.d, ntx, ntiles, c.in_prev >= 0 ? 1 : 0, g->ctl, mc, mp, mr, pool[c.out_cur],
-      c.out_prev >= 0 ? pool[c.out_prev] : nullptr, prm, g->partials, g->partials_stride, g->counters);
+  th_launch(k_cheb_tb<LM, EY, ST, SC, LA, FI>, nblk, dim3(TB_EX, EY), smem, st, P.d, ntx, ntiles,
+            c.in_prev >= 0 ? 1 : 0, g->ctl, mc, mp, mr, pool[c.out_cur],
+            c.out_prev >= 0 ? pool[c.out_prev] : nullptr, prm, g->partials, g->partials_stride, g->counters);
   TH_CHECK_LAUNCH();
   return TH_OK;
 }
@@ -706,9 +706,9 @@ static th_status tbf_launch(const Plan& P, const VecSet<float>& V, cudaStream_t 
   TH_CUDA(cudaFuncSetAttribute(k_cheb_tbf<LM, ST, LA, FI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int nblk = std::min(ntiles, sm_count());
   if (nblk > g->partials_stride) return th_fail(TH_ESTATE, "partials buffer smaller than the temporal-blocking grid");
-  th_launch(k_cheb_tbf<LM, ST, LA, FI>, nblk, dim3(TB_EX, TBF_EY), smem, st, 
-      P.d, ntx, ntiles, c.in_prev >= 0 ? 1 : 0, g->ctl, mc, mp, mr, mx, my, mz, g->invd32, pool[c.out_cur],
-      c.out_prev >= 0 ? pool[c.out_prev] : nullptr, prm, g->partials, g->partials_stride, g->counters);
+  th_launch(k_cheb_tbf<LM, ST, LA, FI>, nblk, dim3(TB_EX, TBF_EY), smem, st, P.d, ntx, ntiles,
+            c.in_prev >= 0 ? 1 : 0, g->ctl, mc, mp, mr, mx, my, mz, g->invd32, pool[c.out_cur],
+            c.out_prev >= 0 ? pool[c.out_prev] : nullptr, prm, g->partials, g->partials_stride, g->counters);
   TH_CHECK_LAUNCH();
   return TH_OK;
 }
@@ -811,9 +811,8 @@ static th_status enq_cheb_tail(const Plan& P, const VecSet<TV>& V, const TC* gx,
       if (P.v4) {
 #define TH_CHEB4(SC, LA)                                                                                     \
   TH_UNI(P.uni && tc_f32,                                                                                    \
-         th_launch(k_cheb_v4<TC, SC, LA, U>, P.gb4, P.tb4, 0, st, P.d, P.zc, g->ctl, gx, gy, gz, g->tab, V.r, zprev, \
-                                                           zcur, znext, c1, c2, g->partials,                  \
-                                                           g->partials_stride, g->counters))
+         th_launch(k_cheb_v4<TC, SC, LA, U>, P.gb4, P.tb4, 0, st, P.d, P.zc, g->ctl, gx, gy, gz, g->tab,     \
+                   V.r, zprev, zcur, znext, c1, c2, g->partials, g->partials_stride, g->counters))
         if (P.scaled) {
           if (last) TH_CHEB4(true, true); else TH_CHEB4(true, false);
         } else {
@@ -826,8 +825,8 @@ static th_status enq_cheb_tail(const Plan& P, const VecSet<TV>& V, const TC* gx,
     }
     if constexpr (sizeof(TV) == 8) {  // plain FP64 path: expanded form with the stored diagonal
 #define TH_CHEB64(SC, LA)                                                                                    \
-  th_launch(k_cheb64x<SC, LA>, P.gb, P.tb, 0, st, P.d, g->ctl, g->f64, g->dg64, V.r, zprev, zcur, znext, V.invd, c1, c2, \
-                                           g->partials, g->partials_stride, g->counters)
+  th_launch(k_cheb64x<SC, LA>, P.gb, P.tb, 0, st, P.d, g->ctl, g->f64, g->dg64, V.r, zprev, zcur, znext,     \
+            V.invd, c1, c2, g->partials, g->partials_stride, g->counters)
       if (P.scaled) {
         if (last) TH_CHEB64(true, true); else TH_CHEB64(true, false);
       } else {
@@ -838,8 +837,8 @@ static th_status enq_cheb_tail(const Plan& P, const VecSet<TV>& V, const TC* gx,
       continue;
     }
 #define TH_CHEB(SC, LA)                                                                                      \
-  th_launch(k_cheb<TV, TC, SC, LA>, P.gb, P.tb, 0, st, P.d, g->ctl, gx, gy, gz, g->tab, V.r, zprev, zcur, znext, \
-                                                V.invd, c1, c2, g->partials, g->partials_stride, g->counters)
+  th_launch(k_cheb<TV, TC, SC, LA>, P.gb, P.tb, 0, st, P.d, g->ctl, gx, gy, gz, g->tab, V.r, zprev, zcur,    \
+            znext, V.invd, c1, c2, g->partials, g->partials_stride, g->counters)
     if (P.scaled) {
       if (last) TH_CHEB(true, true); else TH_CHEB(true, false);
     } else {
@@ -871,7 +870,7 @@ static th_status enq_precond_tail(const Plan& P, const VecSet<TV>& V, cudaStream
   }
   if (P.pc == TH_PC_ZLINE) {
     th_launch(k_zline<TV>, P.gcol, P.tb, 0, st, P.d, g->ctl, g->f32.gz, g->zl_m, g->zl_c, V.r, V.zc[0], g->partials,
-                                         g->partials_stride, g->counters);
+              g->partials_stride, g->counters);
     TH_CHECK_LAUNCH();
   }
   return TH_OK;
@@ -884,16 +883,15 @@ static th_status enq_iteration(const Plan& P, const VecSet<TV>& V, cudaStream_t 
   thermal_grid* g = P.g;
   TV* zf = z_final(P, V);
   if constexpr (sizeof(TV) == 8) {
-    th_launch(k_spmv_dot64x<>, P.gb, P.tb, 0, st, P.d, g->ctl, g->f64, g->dg64, zf, V.p[parity], V.p[1 - parity], V.mu,
-                                         g->partials, g->partials_stride, g->counters);
+    th_launch(k_spmv_dot64x<>, P.gb, P.tb, 0, st, P.d, g->ctl, g->f64, g->dg64, zf, V.p[parity], V.p[1 - parity],
+              V.mu, g->partials, g->partials_stride, g->counters);
   } else if (P.v4) {
-    TH_UNI(P.uni, th_launch(k_spmv_dot_v4<U>, P.nbs4, P.tb4, 0, st, P.d, P.zc, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz,
-                                                           g->tab, zf, V.p[parity], V.p[1 - parity], V.mu,
-                                                           g->partials, g->partials_stride, g->counters));
+    TH_UNI(P.uni, th_launch(k_spmv_dot_v4<U>, P.nbs4, P.tb4, 0, st, P.d, P.zc, g->ctl, g->f32.gx, g->f32.gy,
+                            g->f32.gz, g->tab, zf, V.p[parity], V.p[1 - parity], V.mu, g->partials,
+                            g->partials_stride, g->counters));
   } else {
     th_launch(k_spmv_dot<float, float>, P.gb, P.tb, 0, st, P.d, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz, g->tab, zf,
-                                                    V.p[parity], V.p[1 - parity], V.mu, g->partials,
-                                                    g->partials_stride, g->counters);
+              V.p[parity], V.p[1 - parity], V.mu, g->partials, g->partials_stride, g->counters);
   }
   TH_CHECK_LAUNCH();
   TH_TRY((enq_update<TV, false>(P, V, st, 1 - parity, 1, 0)));
@@ -912,15 +910,14 @@ static void launch_residual_v4(const Plan& P, cudaStream_t st, const float* nh, 
   thermal_grid* g = P.g;
   const TP* const* pt = (const TP* const*)g->dev_ptrs;
   if (!uni) {
-    th_launch(k_residual_df_v4<TP, -1, false>, P.nbf4, P.tb4, 0, st, P.d, P.zc, g->ctl, g->tab, g->f32, g->f32lo, g->th_hi,
-                                                              g->th_lo, pt, nh, nl, g->r32, count_outer, ri,
-                                                              g->partials, g->partials_stride, g->counters);
+    th_launch(k_residual_df_v4<TP, -1, false>, P.nbf4, P.tb4, 0, st, P.d, P.zc, g->ctl, g->tab, g->f32, g->f32lo,
+              g->th_hi, g->th_lo, pt, nh, nl, g->r32, count_outer, ri, g->partials, g->partials_stride, g->counters);
     return;
   }
 #define TH_RES4(ZI)                                                                                           \
-  th_launch(k_residual_df_v4<TP, ZI, true>, P.nbq4, P.tb4, 0, st, P.d, P.zc, g->ctl, g->tab, g->f32, g->f32lo, g->th_hi, \
-                                                          g->th_lo, pt, nh, nl, g->r32, count_outer, ri,        \
-                                                          g->partials, g->partials_stride, g->counters)
+  th_launch(k_residual_df_v4<TP, ZI, true>, P.nbq4, P.tb4, 0, st, P.d, P.zc, g->ctl, g->tab, g->f32,         \
+            g->f32lo, g->th_hi, g->th_lo, pt, nh, nl, g->r32, count_outer, ri, g->partials,                  \
+            g->partials_stride, g->counters)
   switch (zi) {
     case 0: TH_RES4(0); break;
     case 1: TH_RES4(1); break;
@@ -956,23 +953,22 @@ static th_status enq_residual(const Plan& P, cudaStream_t st, int mode, int coun
       return TH_OK;
     }
     if (P.pdtype == TH_F32)
-      TH_UNI(P.uni, th_launch(k_residual_df<float, U>, P.gb, P.tb, 0, st, 
-                        P.d, g->ctl, g->f32, g->f32lo, g->tab, g->th_hi, g->th_lo, (const float* const*)g->dev_ptrs,
-                        nh, nl, g->r32, count_outer, g->partials, g->partials_stride, g->counters));
+      TH_UNI(P.uni, th_launch(k_residual_df<float, U>, P.gb, P.tb, 0, st, P.d, g->ctl, g->f32, g->f32lo, g->tab,
+                              g->th_hi, g->th_lo, (const float* const*)g->dev_ptrs, nh, nl, g->r32, count_outer,
+                              g->partials, g->partials_stride, g->counters));
     else
-      TH_UNI(P.uni, th_launch(k_residual_df<double, U>, P.gb, P.tb, 0, st, 
-                        P.d, g->ctl, g->f32, g->f32lo, g->tab, g->th_hi, g->th_lo,
-                        (const double* const*)g->dev_ptrs, nh, nl, g->r32, count_outer, g->partials,
-                        g->partials_stride, g->counters));
+      TH_UNI(P.uni, th_launch(k_residual_df<double, U>, P.gb, P.tb, 0, st, P.d, g->ctl, g->f32, g->f32lo, g->tab,
+                              g->th_hi, g->th_lo, (const double* const*)g->dev_ptrs, nh, nl, g->r32, count_outer,
+                              g->partials, g->partials_stride, g->counters));
     TH_CHECK_LAUNCH();
     return TH_OK;
   }
   const double* th = g->theta[0];
   const double* thn = P.transient ? g->theta_n : nullptr;
 #define TH_RES(TP, TR, RP)                                                                                     \
-  th_launch(k_residual<TP, TR>, P.gb, P.tb, 0, st, P.d, g->ctl, g->f64, g->tab, th, (const TP*)nullptr,             \
-                                            (const TP* const*)g->dev_ptrs, thn, RP, mode, count_outer,         \
-                                            g->partials, g->partials_stride, g->counters)
+  th_launch(k_residual<TP, TR>, P.gb, P.tb, 0, st, P.d, g->ctl, g->f64, g->tab, th, (const TP*)nullptr,      \
+            (const TP* const*)g->dev_ptrs, thn, RP, mode, count_outer, g->partials, g->partials_stride,      \
+            g->counters)
   if (P.pdtype == TH_F32) {
     if (out64) TH_RES(float, double, g->r64); else TH_RES(float, float, g->r32);
   } else {
@@ -1156,11 +1152,11 @@ static th_status enq_step_copy(const Plan& P, cudaStream_t st) {
       th_launch(k_step_extrap64, nb1(n), 256, 0, st, n, g->theta[0], g->theta_n, g->thm64);
     else
       if (P.extrap_order == 3)
-        th_launch(k_step_extrapq_df_v4<3>, P.nbu4, 256, 0, st, n / 4, g->ctl, g->th_hi, g->th_lo, g->thm_hi, g->thm_lo,
-                                                        g->thm2_hi, g->thm2_lo, g->thm3_hi, g->thm3_lo);
+        th_launch(k_step_extrapq_df_v4<3>, P.nbu4, 256, 0, st, n / 4, g->ctl, g->th_hi, g->th_lo, g->thm_hi,
+                  g->thm_lo, g->thm2_hi, g->thm2_lo, g->thm3_hi, g->thm3_lo);
       else if (P.extrap_order == 2)
-        th_launch(k_step_extrapq_df_v4<2>, P.nbu4, 256, 0, st, n / 4, g->ctl, g->th_hi, g->th_lo, g->thm_hi, g->thm_lo,
-                                                        g->thm2_hi, g->thm2_lo, nullptr, nullptr);
+        th_launch(k_step_extrapq_df_v4<2>, P.nbu4, 256, 0, st, n / 4, g->ctl, g->th_hi, g->th_lo, g->thm_hi,
+                  g->thm_lo, g->thm2_hi, g->thm2_lo, nullptr, nullptr);
       else if (P.v4)
         th_launch(k_step_extrap_df_v4, P.nbu4, 256, 0, st, n / 4, g->th_hi, g->th_lo, g->thm_hi, g->thm_lo);
       else
@@ -1877,59 +1873,57 @@ extern "C" th_status thermal_kernel_time(thermal_grid* g, int kernel, int reps, 
         break;
       case 1:
         if (P.v4) {
-          TH_UNI(uni, th_launch(k_cheb_v4<float, true, false, U>, P.gb4, P.tb4, 0, s, 
-                          P.d, P.zc, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz, g->tab, V.r, V.zc[0], V.zc[1], V.zc[2],
-                          c1, c2, g->partials, g->partials_stride, g->counters));
+          TH_UNI(uni, th_launch(k_cheb_v4<float, true, false, U>, P.gb4, P.tb4, 0, s, P.d, P.zc, g->ctl, g->f32.gx,
+                                g->f32.gy, g->f32.gz, g->tab, V.r, V.zc[0], V.zc[1], V.zc[2], c1, c2, g->partials,
+                                g->partials_stride, g->counters));
           break;
         }
-        th_launch(k_cheb<float, float, true, false>, P.gb, P.tb, 0, s, P.d, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz, g->tab,
-                                                                V.r, V.zc[0], V.zc[1], V.zc[2], V.invd, c1, c2,
-                                                                g->partials, g->partials_stride, g->counters);
+        th_launch(k_cheb<float, float, true, false>, P.gb, P.tb, 0, s, P.d, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz,
+                  g->tab, V.r, V.zc[0], V.zc[1], V.zc[2], V.invd, c1, c2, g->partials, g->partials_stride,
+                  g->counters);
         break;
       case 2:
         if (P.v4) {
-          th_launch(k_cheb_v4<__nv_bfloat16, true, false, false>, P.gb4, P.tb4, 0, s, 
-              P.d, P.zc, g->ctl, g->f16.gx, g->f16.gy, g->f16.gz, g->tab, V.r, V.zc[0], V.zc[1], V.zc[2], c1, c2,
-              g->partials, g->partials_stride, g->counters);
+          th_launch(k_cheb_v4<__nv_bfloat16, true, false, false>, P.gb4, P.tb4, 0, s, P.d, P.zc, g->ctl, g->f16.gx,
+                    g->f16.gy, g->f16.gz, g->tab, V.r, V.zc[0], V.zc[1], V.zc[2], c1, c2, g->partials,
+                    g->partials_stride, g->counters);
           break;
         }
-        th_launch(k_cheb<float, __nv_bfloat16, true, false>, P.gb, P.tb, 0, s, 
-            P.d, g->ctl, g->f16.gx, g->f16.gy, g->f16.gz, g->tab, V.r, V.zc[0], V.zc[1], V.zc[2], V.invd, c1, c2,
-            g->partials, g->partials_stride, g->counters);
+        th_launch(k_cheb<float, __nv_bfloat16, true, false>, P.gb, P.tb, 0, s, P.d, g->ctl, g->f16.gx, g->f16.gy,
+                  g->f16.gz, g->tab, V.r, V.zc[0], V.zc[1], V.zc[2], V.invd, c1, c2, g->partials, g->partials_stride,
+                  g->counters);
         break;
       case 3:
         if (P.v4) {
-          TH_UNI(uni, th_launch(k_spmv_dot_v4<U>, P.nbs4, P.tb4, 0, s, P.d, P.zc, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz,
-                                                              g->tab, V.zc[0], V.p[0], V.p[1], V.mu, g->partials,
-                                                              g->partials_stride, g->counters));
+          TH_UNI(uni, th_launch(k_spmv_dot_v4<U>, P.nbs4, P.tb4, 0, s, P.d, P.zc, g->ctl, g->f32.gx, g->f32.gy,
+                                g->f32.gz, g->tab, V.zc[0], V.p[0], V.p[1], V.mu, g->partials, g->partials_stride,
+                                g->counters));
           break;
         }
         th_launch(k_spmv_dot<float, float>, P.gb, P.tb, 0, s, P.d, g->ctl, g->f32.gx, g->f32.gy, g->f32.gz, g->tab,
-                                                       V.zc[0], V.p[0], V.p[1], V.mu, g->partials,
-                                                       g->partials_stride, g->counters);
+                  V.zc[0], V.p[0], V.p[1], V.mu, g->partials, g->partials_stride, g->counters);
         break;
       case 4:
         if (P.v4) {
-          TH_UNI(uni, th_launch(k_update_v4<false, 1, U>, P.nbr4, 256, 0, s, P.d.n / 4, g->ctl, V.x, V.p[1], V.r, V.mu,
-                                                                     V.invd, V.zc[0], 1.0f, 1, 1, 0, g->partials,
-                                                                     g->partials_stride, g->counters, P.d, g->tab));
+          TH_UNI(uni, th_launch(k_update_v4<false, 1, U>, P.nbr4, 256, 0, s, P.d.n / 4, g->ctl, V.x, V.p[1], V.r,
+                                V.mu, V.invd, V.zc[0], 1.0f, 1, 1, 0, g->partials, g->partials_stride, g->counters,
+                                P.d, g->tab));
           break;
         }
-        th_launch(k_update<float, false, 1>, P.gb, P.tb, 0, s, P.d, g->ctl, V.x, V.p[1], V.r, V.mu, V.invd, V.zc[0], 1.0f,
-                                                        1, 1, 0, g->partials, g->partials_stride, g->counters);
+        th_launch(k_update<float, false, 1>, P.gb, P.tb, 0, s, P.d, g->ctl, V.x, V.p[1], V.r, V.mu, V.invd, V.zc[0],
+                  1.0f, 1, 1, 0, g->partials, g->partials_stride, g->counters);
         break;
       case 5:
         th_launch(k_residual<float, float>, P.gb, P.tb, 0, s, P.d, g->ctl, g->f64, g->tab, g->theta[0], nullptr,
-                                                       (const float* const*)g->dev_ptrs,
-                                                       P.transient ? g->theta_n : nullptr, g->r32, 2, 0,
-                                                       g->partials, g->partials_stride, g->counters);
+                  (const float* const*)g->dev_ptrs, P.transient ? g->theta_n : nullptr, g->r32, 2, 0, g->partials,
+                  g->partials_stride, g->counters);
         break;
       case 6:
         k_apply64x<<<P.gb, P.tb, 0, s>>>(P.d, g->f64, g->dg64, g->zc64[0], g->zc64[1]);
         break;
       case 7:
-        th_launch(k_cheb64x<true, false>, P.gb, P.tb, 0, s, P.d, g->ctl, g->f64, g->dg64, W.r, W.zc[0], W.zc[1], W.zc[2],
-                                                     W.invd, 0.5, 0.5, g->partials, g->partials_stride, g->counters);
+        th_launch(k_cheb64x<true, false>, P.gb, P.tb, 0, s, P.d, g->ctl, g->f64, g->dg64, W.r, W.zc[0], W.zc[1],
+                  W.zc[2], W.invd, 0.5, 0.5, g->partials, g->partials_stride, g->counters);
         break;
       default:
         if (P.v4) {
@@ -1937,10 +1931,10 @@ extern "C" th_status thermal_kernel_time(thermal_grid* g, int kernel, int reps, 
                                     -1, ResidInit{}, uni);
           break;
         }
-        TH_UNI(uni, th_launch(k_residual_df<float, U>, P.gb, P.tb, 0, s, 
-                        P.d, g->ctl, g->f32, g->f32lo, g->tab, g->th_hi, g->th_lo, (const float* const*)g->dev_ptrs,
-                        P.transient ? g->thn_hi : nullptr, P.transient ? g->thn_lo : nullptr, g->r32, 0,
-                        g->partials, g->partials_stride, g->counters));
+        TH_UNI(uni, th_launch(k_residual_df<float, U>, P.gb, P.tb, 0, s, P.d, g->ctl, g->f32, g->f32lo, g->tab,
+                              g->th_hi, g->th_lo, (const float* const*)g->dev_ptrs, P.transient ? g->thn_hi : nullptr,
+                              P.transient ? g->thn_lo : nullptr, g->r32, 0, g->partials, g->partials_stride,
+                              g->counters));
         break;
     }
     TH_CHECK_LAUNCH();
