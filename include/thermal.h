@@ -106,8 +106,9 @@ typedef struct thermal_solve_opts {
   int cheb_fuse;       /* Chebyshev steps per launch (temporal blocking) on grids with       */
                        /* nx % 4 == 0: layer table up to 12 layers, per-face arrays up to 8   */
                        /* (not with the BF16 coefficients): 0 auto (small layer-table grids,  */
-                       /* any nx: the whole inner solve in one launch; else 4), 1 one step    */
-                       /* per launch, 2..4 (0)                                                */
+                       /* any nx with FP32 coefficients: the whole inner solve in one launch  */
+                       /* where the stream's SMs hold it; else 4), 1 one step per launch,     */
+                       /* 2..4 (0)                                                            */
   int ad_check;        /* ADAPTIVE: PCG iterations between true-residual evaluations of the   */
                        /* switching criterion, rounded up to even; 0: 20 steady, 6 transient  */
                        /* (the paper's 20 and 5 on the two-iteration loop body) (0)           */

@@ -579,6 +579,7 @@ th_status grid_ensure_workspace(thermal_grid* g, bool need64, cudaStream_t s) {
     g->wait_lost = (int*)&((CtlBox*)g->ctl_host)->wait_lost;  // the word stands where the device has its address
     *g->wait_lost = 0;
     TH_CUDA(cudaMemcpyAsync(&box->wait_lost, &g->wait_lost, sizeof(int*), cudaMemcpyHostToDevice, s));
+    TH_CUDA(cudaStreamSynchronize(s));  // ready for any stream, also if this call fails later on
     g->ws32 = true;
   }
   if (need64 && !g->ws64) {

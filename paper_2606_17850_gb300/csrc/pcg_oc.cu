@@ -117,7 +117,7 @@ static size_t oc_bytes(const thermal_grid* g) {
   return sizeof(OCWord) * (2 * (size_t)device_sms() + 1 + 2 * (size_t)oc_column_words(lmax) * g->nx * g->ny);
 }
 
-// workspace of oc_run, before any graph capture
+// workspace of oc_run, before any graph capture; ready for any stream when this returns
 th_status oc_prepare(thermal_grid* g, cudaStream_t s) {
   if (g->oc_sync) return TH_OK;
   if (cudaMalloc(&g->oc_sync, oc_bytes(g)) != cudaSuccess) {
@@ -125,8 +125,12 @@ th_status oc_prepare(thermal_grid* g, cudaStream_t s) {
     g->oc_sync = nullptr;
     return th_fail(TH_ENOMEM, "exchange allocation failed");
   }
-  TH_CUDA(cudaMemsetAsync(g->oc_sync, 0, oc_bytes(g), s));
-  return TH_OK;
+  cudaError_t e = cudaMemsetAsync(g->oc_sync, 0, oc_bytes(g), s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) return TH_OK;
+  cudaFree(g->oc_sync);  // not cleared: not the grid's
+  g->oc_sync = nullptr;
+  return th_fail(TH_ECUDA, "clearing the exchange words failed: %s", cudaGetErrorString(e));
 }
 
 th_status oc_run(thermal_grid* g, const OCRun& o, cudaStream_t s) {
