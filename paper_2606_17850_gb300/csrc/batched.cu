@@ -354,7 +354,7 @@ __device__ __forceinline__ MGDev mg_dev(const MGBDesc& D, int k, int L) {
 // path), instances of different depths in the same phases; the last pass also reduces
 // r^T z.  A level is two phases on shared-memory tiles (mg_tile.cuh); with a phase each
 // for smoothing and restriction, every column reading its neighbours' from global memory,
-// the 32 stacks of 128^2 x 4 to 512^2 x 8 took 147 ms, now 76 ms.
+// the 32 stacks of 128^2 x 4 to 512^2 x 8 took 147 ms, now 73 ms.
 __device__ void mg_vcycle_batched(const BArgs& A, cg::grid_group& grid) {
   __shared__ double red[32];
   __shared__ MGUni<8> tab;
@@ -445,7 +445,7 @@ __device__ void mg_vcycle_batched(const BArgs& A, cg::grid_group& grid) {
 // registers (measured: 0.92 s vs 1.12 s with two blocks per SM for the 64 stacks).
 // MGP: the multigrid instantiation (its V-cycle phases are compiled only there, so
 // the other preconditioners keep their register allocation); four blocks per SM there (its
-// tile passes wait on latency: 32 stacks 91.6 / 76.2 / 74.3 ms at 2 / 3 / 4 blocks)
+// tile passes wait on latency: 32 stacks 91.6 / 76.2 / 74.3 ms at 2 / 3 / 4 blocks when chosen)
 template <typename TP, bool MGP>
 __global__ void __launch_bounds__(TH_BX* TH_BY4, MGP ? 4 : 3) k_batched(BArgs A) {
   cg::grid_group grid = cg::this_grid();

@@ -12,8 +12,8 @@
 // exchange cost.  No tensor copies, so any nx.
 //
 // Measured (before: one launch per chunk of four steps where nx % 4 == 0, else per step):
-// steady 64 x 64 x 4, degree 30, in a graph 2.24 -> 0.80 ms; steady 301 x 203 x 8 36.4 ->
-// 5.7 ms; one 130 x 70 x 4 time step 0.86 -> 0.30 ms.  What bounds it now is shared memory
+// steady 64 x 64 x 4, degree 30, in a graph 2.24 -> 0.76 ms; steady 301 x 203 x 8 36.4 ->
+// 5.8 ms; one 130 x 70 x 4 time step 0.86 -> 0.30 ms.  What bounds it now is shared memory
 // and issue inside a step (32 rows x 8 layers: 0.67 us for 1280 wavefronts) and the
 // latency of 1.5 us per exchange or sum.
 //
@@ -24,11 +24,12 @@
 // an exchange 8 us: the instructions of all its threads, not the latency.)  A dot product
 // is summed the same way: each CTA writes its FP64 partial as one word into a slot of its
 // own, warp 0 of every CTA reads all slots and adds them in slot order, so all CTAs hold
-// the same total, deterministically.  Two sets of words alternate, and exchanges and sums are numbered
-// apart: a CTA writes a set again only after it has read its neighbours' words of the
-// exchange in between (everybody's of the sum in between), which they wrote after they had
-// read the earlier ones.  Waits are bounded (one second), after which the error is
-// recorded and every CTA leaves.
+// the same total, deterministically.  Two sets of words alternate, and exchanges and sums
+// are numbered apart: a CTA writes a set again only after it has read its neighbours' words
+// of the exchange in between (everybody's of the sum in between), which they wrote after
+// they had read the earlier ones.  Waits are bounded (one second), after which the error is
+// recorded and every CTA leaves; the cooperative launch starts no CTA before all of them have
+// a place, however long other work holds the SMs.
 #pragma once
 
 #include "kernels_tb.cuh"

@@ -1758,8 +1758,8 @@ static th_status precond_once(thermal_grid* g, double dt, const thermal_solve_op
   // Fused chunks and the V-cycle read nothing but r: they take it from the caller's buffer
   // and leave z in the caller's (16-byte aligned, as the tensor copies and 4-cell loads
   // want), without the start of an inner solve and the two copies.  Chebyshev-29 on
-  // 1024 x 1024 x 8: 365 -> 318 us, a V-cycle on 640 x 384 x 8 130 -> 102 us, Chebyshev-16
-  // on a 500 x 333 x 6 conductivity map 162 -> 127 us.
+  // 1024 x 1024 x 8: 365 -> 323 us, a V-cycle on 640 x 384 x 8 130 -> 103 us, Chebyshev-16
+  // on a 500 x 333 x 6 conductivity map 162 -> 132 us.
   if (direct == 2 && (P.fused || P.pc == TH_PC_MG)) {
     V.r = const_cast<float*>(r);
     if (P.pc == TH_PC_CHEB && P.zfin == 3) V.mu = z;
