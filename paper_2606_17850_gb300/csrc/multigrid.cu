@@ -140,6 +140,14 @@ constexpr size_t mg_xs_bytes() {
   return sizeof(float) * LMAX * MGT_EX * MG_EY;
 }
 
+// Row of tiles: more than 65535 of them (ny from 393211) continue in z; those past the last
+// hold no column.  (Tiles in one grid dimension, with a division, cost a 1024^2 x 10 cycle 2 %.)
+__device__ __forceinline__ int mg_tile_y() { return (int)(blockIdx.y + gridDim.y * blockIdx.z); }
+dim3 mg_tile_grid(int nx, int ny) {
+  const unsigned rows = (ny + MG_EY - 3) / (MG_EY - 2), z = (rows + 65534) / 65535;
+  return dim3((nx + MGT_EX - 3) / (MGT_EX - 2), (rows + z - 1) / z, z);
+}
+
 template <int LMAX, bool UNI>
 __global__ void __launch_bounds__(MGT_EX* MG_EY, LMAX <= 12 ? MG_MINB : 1)
     k_mg_down(const Ctl* ctl, MGDev v, const __grid_constant__ MGUni<LMAX> U, const float* __restrict__ b,
@@ -147,7 +155,7 @@ __global__ void __launch_bounds__(MGT_EX* MG_EY, LMAX <= 12 ? MG_MINB : 1)
   grid_dep_enter();
   if (ld_int(&ctl->done)) return;
   extern __shared__ __align__(16) float mg_xs[];
-  mgt_down<LMAX, UNI, MG_EY, false>(v, U, blockIdx.x, blockIdx.y, b, x, nxc, nyc, bc, mg_xs);
+  mgt_down<LMAX, UNI, MG_EY, false>(v, U, blockIdx.x, mg_tile_y(), b, x, nxc, nyc, bc, mg_xs);
 }
 
 // way up; on the finest level (RZ) with r^T z and beta (b is r)
@@ -160,7 +168,7 @@ __global__ void __launch_bounds__(MGT_EX* MG_EY, LMAX <= 12 ? MG_MINB : 1)
   if (ld_int(&ctl->done)) return;
   extern __shared__ __align__(16) float mg_xs[];
   if (!RZ) {
-    mgt_up<LMAX, UNI, MG_EY, false, RZ>(v, U, blockIdx.x, blockIdx.y, b, xin, xc, nxc, nyc, xout, mg_xs);
+    mgt_up<LMAX, UNI, MG_EY, false, RZ>(v, U, blockIdx.x, mg_tile_y(), b, xin, xc, nxc, nyc, xout, mg_xs);
     return;
   }
   // the tiles over the blocks that are resident at once, so that the reduction's tail (7 us
@@ -710,7 +718,7 @@ static th_status mg_half(thermal_grid* g, int k, bool up, const float* b, float*
   const MGHier* h = g->mg;
   const MGLevelH &l = h->lv[k], &c = h->lv[k + 1];
   const MGUni<LMAX> U = uni_of<LMAX>(h, k);
-  const dim3 gr((l.nx + MGT_EX - 3) / (MGT_EX - 2), (l.ny + MG_EY - 3) / (MG_EY - 2)), bl(MGT_EX, MG_EY);
+  const dim3 gr = mg_tile_grid(l.nx, l.ny), bl(MGT_EX, MG_EY);
   constexpr size_t sm = mg_xs_bytes<LMAX>();
   static_assert(sm <= (40u << 10), "a tile needs the opt-in for larger shared memory");
   auto launch = [&](auto* kern, dim3 blocks, auto... a) -> th_status {
@@ -720,7 +728,8 @@ static th_status mg_half(thermal_grid* g, int k, bool up, const float* b, float*
   };
   if (!up) return launch(k_mg_down<LMAX, UNI>, gr, g->ctl, dev_of(l, g->L), U, b, x, c.nx, c.ny, c.b);
   if (k == 0)
-    return launch(k_mg_up<LMAX, UNI, true>, std::min(gr.x * gr.y, (LMAX <= 12 ? MG_MINB : 1u) * device_sms()), g->ctl,
+    return launch(k_mg_up<LMAX, UNI, true>,
+                  std::min(mgt_tiles<MG_EY>(l.nx, l.ny), (LMAX <= 12 ? (int)MG_MINB : 1) * device_sms()), g->ctl,
                   dev_of(l, g->L), U, b, x, xc, c.nx, c.ny, z, g->partials, g->partials_stride, g->counters);
   return launch(k_mg_up<LMAX, UNI, false>, gr, g->ctl, dev_of(l, g->L), U, b, x, xc, c.nx, c.ny, z, g->partials,
                 g->partials_stride, g->counters);

@@ -1342,3 +1342,16 @@ def test_streaming_sizes_are_streamed():
                        (1028, 520, "l6"), (1084, 700, "l5"), (772, 768, "c2")):
         assert pays(nx, ny, STACKS[mk]().L), (nx, ny, mk)
     assert not pays(76, 37, 8) and not pays(128, 128, 4) and not pays(1024, 1024, 10) and not pays(1023, 1024, 8)
+
+
+@pytest.mark.parametrize("n_long,n_short,L", [(400001, 3, 2), (524280, 1, 1)])
+def test_mg_vcycle_on_long_grids(n_long, n_short, L):
+    """As many rows as the layered kernels' grids reach (ny / 8 <= 65535): the V-cycle of a
+    tall grid is that of the wide one with x and y exchanged (square cells), up to the order
+    of FP32 additions, with the bound of test_mg_vcycle_matches_oracle."""
+    st = ti.Stack(tuple(ti.si() if i % 2 == 0 else ti.cu(200.0) for i in range(L)), h=1e4)
+    r = ti.random_vector(n_long * n_short * L, 5).astype(np.float32).reshape(L, n_long, n_short)
+    tall = grid_of(n_short, n_long, st).precond(cuda(r.ravel()), 0.0, precond="mg").reshape(L, n_long, n_short)
+    wide = grid_of(n_long, n_short, st).precond(cuda(np.ascontiguousarray(r.transpose(0, 2, 1)).ravel()), 0.0,
+                                                precond="mg").reshape(L, n_short, n_long).transpose(1, 2)
+    assert (tall - wide).abs().max().item() <= 2e-5 * wide.abs().max().item()
