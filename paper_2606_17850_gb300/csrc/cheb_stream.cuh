@@ -22,25 +22,13 @@ static th_status st_launch(thermal_grid* g, const Dims& d, const StreamChunk& c,
   const LayerTab& T = g->tab_host;
   const int L = d.L;
   for (int z = 0; z < L; ++z) {
-    const float sz = T.s32[z], gx = T.gxl[z], gy = T.gyl[z];
-    const float gzu = (z + 1 < L) ? T.gzl[z] : 0.f, gzd = (z > 0) ? T.gzl[z - 1] : 0.f;
-    prm.gx[z] = two(gx);
-    prm.gy[z] = two(gy);
-    prm.gzu[z] = two(gzu);
-    prm.gzd[z] = two(gzd);
-    // diagonal summed in the one-step kernels' order: s, +x, -x, +y, -y, +z, -z
-    for (int nyf = 0; nyf < 3; ++nyf)
-      for (int nxf = 0; nxf < 3; ++nxf) {
-        float dg = sz;
-        dg += nxf >= 1 ? gx : 0.f;
-        dg += nxf >= 2 ? gx : 0.f;
-        dg += nyf >= 1 ? gy : 0.f;
-        dg += nyf >= 2 ? gy : 0.f;
-        dg += gzu;
-        dg += gzd;
-        prm.invd[nxf + 3 * nyf][z] = 1.0f / dg;
-        if (nxf == 2 && nyf == 2) prm.nd[z] = two(-dg);
-      }
+    const LayerCoefs q = layer_coefs(T, L, z);
+    prm.gx[z] = two(q.gx);
+    prm.gy[z] = two(q.gy);
+    prm.gzu[z] = two(q.gzu);
+    prm.gzd[z] = two(q.gzd);
+    prm.nd[z] = two(-q.d);
+    for (int k = 0; k < 9; ++k) prm.invd[k][z] = q.invd[k];
   }
   CUtensorMap mc, mp, mr;
   std::memset(&mc, 0, sizeof(mc));

@@ -488,6 +488,22 @@ th_status grid_ensure_tab(thermal_grid* g, double dt, cudaStream_t s) {
   return TH_OK;
 }
 
+LayerCoefs layer_coefs(const LayerTab& T, int L, int z) {
+  LayerCoefs c;
+  auto full = [](float hi, float lo) { return (double)hi + (double)lo; };
+  c.gx = T.gxl[z];
+  c.gy = T.gyl[z];
+  c.gzu = z + 1 < L ? T.gzl[z] : 0.f;
+  c.gzd = z > 0 ? T.gzl[z - 1] : 0.f;
+  c.s = T.s32[z];
+  c.d = (float)((double)c.s + 2.0 * c.gx + 2.0 * c.gy + c.gzu + c.gzd);
+  const double gx = full(T.gxl_hi[z], T.gxl_lo[z]), gy = full(T.gyl_hi[z], T.gyl_lo[z]);
+  const double gz = (z + 1 < L ? full(T.gzl_hi[z], T.gzl_lo[z]) : 0.0) +
+                    (z > 0 ? full(T.gzl_hi[z - 1], T.gzl_lo[z - 1]) : 0.0);
+  for (int k = 0; k < 9; ++k) c.invd[k] = (float)(1.0 / (T.s64[z] + (k % 3) * gx + (k / 3) * gy + gz));
+  return c;
+}
+
 th_status grid_ensure_qd(thermal_grid* g, double dt, cudaStream_t s) {
   TH_TRY(grid_ensure_tab(g, dt, s));
   const double key = dt > 0.0 ? dt : 0.0;

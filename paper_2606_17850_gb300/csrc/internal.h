@@ -229,6 +229,16 @@ void graph_cache_free(GraphCache* c);
 // Lanczos interval and the Chebyshev three-term coefficients (c1[m], c2[m], m < k).
 th_status solver_cheb_coeffs(thermal_grid* g, double dt, const thermal_solve_opts* o, std::vector<float>& c1,
                              std::vector<float>& c2, float* inv_theta, double* lmin, double* lmax, cudaStream_t s);
+// Coefficients of one layer of a layer-uniform grid for the fused Chebyshev kernels: FP32
+// faces (0 where there is none) and sink + capacity term; the diagonal of a cell with all
+// four in-plane faces as the FP32 number nearest to the sum of these, so that the expanded
+// product r - d v + sum_f g_f v_f loses least where v is smooth; and the inverse diagonals by
+// (x faces present) + 3 (y faces present), rounded once from the FP64 faces as the per-cell
+// array is.
+struct LayerCoefs {
+  float gx, gy, gzu, gzd, s, d, invd[9];
+};
+LayerCoefs layer_coefs(const LayerTab& T, int L, int z);
 int device_sms();
 // SMs that kernels launched on s can run on: fewer than the device's in a green context.
 int stream_sms(cudaStream_t s);

@@ -4,9 +4,8 @@
 // iteration with a degree-30 polynomial was ten launches of 6 to 8 us each, of which a
 // fused chunk computes for about 3.  Here one cooperative kernel runs the whole inner
 // solve.  Every CTA owns one tile of (32 - 2H) x (EY - 2H) columns (all layers) grown by
-// H cells; a thread keeps its column's z_m, z_{m-1}, D^-1 r and 1/D in registers (layer
-// pairs, as in kernels_tb.cuh, with the same step arithmetic) and r, x, p in its own
-// shared-memory slots.  H Chebyshev steps run between two exchanges, in which the tile's
+// H cells; a thread keeps its column's z_m, z_{m-1}, r and 1/D in registers (layer pairs, as
+// in kernels_tb.cuh) and r, x, p in its own shared-memory slots.  H Chebyshev steps run between two exchanges, in which the tile's
 // H outermost cells go to the neighbours' halo columns.  With fewer tiles than SMs the
 // halo that is recomputed costs nothing; oc_shape picks EY and H from what a step and an
 // exchange cost.  No tensor copies, so any nx.
@@ -200,7 +199,11 @@ __device__ __forceinline__ bool oc_sum(OCShared& sh, OCWord* sync, int cap, unsi
 // DIFF takes the steps' product in difference form, sum_f g_f (v_f - v), instead of the
 // expanded form: six more additions per cell, for grids that had no fused chunks before
 // (nx % 4 != 0, one difference-form launch per step), so that their vectors are as
-// accurate as they were (4e-8 to 9e-8 of ||z|| against 1.5e-7 in expanded form).
+// accurate as they were.  The residual r - A v is formed before it is scaled: with D^-1 r
+// kept in r's place (one instruction less in difference form, 0.8 % of an iteration) the
+// error against 64 bits was 1.08 times the one-step kernels' in the mean over 1700 grids,
+// degrees and stacks with nx % 4 != 0, and 1.01 times the tiles' elsewhere; it is 1.016 and
+// 0.79 times (what is left of the former: they divide by the diagonal).
 template <int LMAX, int EY, bool DIFF>
 __global__ void __launch_bounds__(TB_EX * EY, 1)
     k_pcg_oc(Dims d, int ntx, int H, int solve, Ctl* ctl, const float* __restrict__ r, float* __restrict__ x_out,
@@ -241,7 +244,7 @@ __global__ void __launch_bounds__(TB_EX * EY, 1)
   // this column's words of the current exchange's set
   OCWord* const col0 = sync + 2 * cap + 1 + (inside ? gx + (long long)d.nx * gy : 0);
   const long long set1 = (long long)oc_column_words(LMAX) * d.pxy;
-  float2 za[LP], zb[LP], iv[LP], rs[LP];  // iv = 1/D, rs = D^-1 r
+  float2 za[LP], zb[LP], iv[LP], rs[LP];  // iv = 1/D, rs = r
 #pragma unroll
   for (int k = 0; k < LP; ++k) {
     float2 rv = make_float2(0.f, 0.f);
@@ -287,8 +290,9 @@ __global__ void __launch_bounds__(TB_EX * EY, 1)
           const float2 dn = k > 0 ? C[k > 0 ? k - 1 : k] : make_float2(0.f, C[LP - 1].x);
           a = __ffma2_rn(P.gzu[k], __fadd2_rn(up, nv), a);  // the faces at the ends are 0
           a = __ffma2_rn(P.gzd[k], __fadd2_rn(dn, nv), a);
-        } else {  // the operation order of k_cheb_tb with every sign turned
-          a = __fmul2_rn(P.nd[k], v);
+          a = __fadd2_rn(rs[k], a);
+        } else {  // the operation order of k_cheb_tb with every sign turned, from r on
+          a = __ffma2_rn(P.nd[k], v, rs[k]);
           a = __ffma2_rn(P.gx[k], __fadd2_rn(q[oR], q[oL]), a);
           a = __ffma2_rn(P.gy[k], __fadd2_rn(q[oU], q[oD]), a);
           if (k + 1 < LP) a = __ffma2_rn(P.gzu[k], C[k + 1 < LP ? k + 1 : k], a);
@@ -296,7 +300,7 @@ __global__ void __launch_bounds__(TB_EX * EY, 1)
           if (k > 0) a = __ffma2_rn(P.gzd[k], C[k > 0 ? k - 1 : k], a);
           else a.y = fmaf(P.gzd[0].y, C[LP - 1].x, a.y);
         }
-        const float2 res = __ffma2_rn(iv[k], a, rs[k]);
+        const float2 res = __fmul2_rn(a, iv[k]);
         N[k] = __ffma2_rn(c2, res, __ffma2_rn(c1, __ffma2_rn(N[k], m1, v), v));
       }
     }
@@ -315,8 +319,8 @@ __global__ void __launch_bounds__(TB_EX * EY, 1)
     // ---- z = M^-1 r on the interior
 #pragma unroll
     for (int k = 0; k < LP; ++k) {
-      rs[k] = __fmul2_rn(rs_[k * PL], iv[k]);
-      za[k] = __fmul2_rn(rs[k], make_float2(P.z1s, P.z1s));
+      rs[k] = rs_[k * PL];
+      za[k] = __fmul2_rn(__fmul2_rn(rs[k], iv[k]), make_float2(P.z1s, P.z1s));
       zb[k] = make_float2(0.f, 0.f);
     }
     int m = 1;

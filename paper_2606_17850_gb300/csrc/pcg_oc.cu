@@ -52,26 +52,14 @@ static th_status oc_launch(thermal_grid* g, const OCRun& o, cudaStream_t s) {
   // layer z is component (z < LMAX/2 ? x : y) of pair z % (LMAX/2)
   auto at = [](float2* a, int z) -> float& { return z < LMAX / 2 ? a[z].x : a[z - LMAX / 2].y; };
   for (int z = 0; z < L; ++z) {
-    const float sz = T.s32[z], gx = T.gxl[z], gy = T.gyl[z];
-    const float gzu = (z + 1 < L) ? T.gzl[z] : 0.f, gzd = (z > 0) ? T.gzl[z - 1] : 0.f;
-    at(prm.gx, z) = gx;
-    at(prm.gy, z) = gy;
-    at(prm.gzu, z) = gzu;
-    at(prm.gzd, z) = gzd;
-    at(prm.s, z) = sz;
-    // diagonal summed in the one-step kernels' order: s, +x, -x, +y, -y, +z, -z
-    for (int nyf = 0; nyf < 3; ++nyf)
-      for (int nxf = 0; nxf < 3; ++nxf) {
-        float dg = sz;
-        dg += nxf >= 1 ? gx : 0.f;
-        dg += nxf >= 2 ? gx : 0.f;
-        dg += nyf >= 1 ? gy : 0.f;
-        dg += nyf >= 2 ? gy : 0.f;
-        dg += gzu;
-        dg += gzd;
-        prm.invd[nxf + 3 * nyf][z] = 1.0f / dg;
-        if (nxf == 2 && nyf == 2) at(prm.nd, z) = -dg;
-      }
+    const LayerCoefs c = layer_coefs(T, L, z);
+    at(prm.gx, z) = c.gx;
+    at(prm.gy, z) = c.gy;
+    at(prm.gzu, z) = c.gzu;
+    at(prm.gzd, z) = c.gzd;
+    at(prm.s, z) = c.s;
+    at(prm.nd, z) = -c.d;
+    for (int q = 0; q < 9; ++q) prm.invd[q][z] = c.invd[q];
   }
   const int tx = TB_EX - 2 * o.shape.halo, ty = EY - 2 * o.shape.halo;
   const int ntx = (d.nx + tx - 1) / tx, nblk = ntx * ((d.ny + ty - 1) / ty), cap = device_sms();

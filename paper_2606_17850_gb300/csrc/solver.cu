@@ -638,25 +638,13 @@ static th_status tb_launch(const Plan& P, const VecSet<float>& V, cudaStream_t s
   // layer z is component (z < LM/2 ? x : y) of pair z % (LM/2)
   auto at = [](float2* a, int z) -> float& { return z < LM / 2 ? a[z].x : a[z - LM / 2].y; };
   for (int z = 0; z < L; ++z) {
-    const float sz = T.s32[z], gx = T.gxl[z], gy = T.gyl[z];
-    const float gzu = (z + 1 < L) ? T.gzl[z] : 0.f, gzd = (z > 0) ? T.gzl[z - 1] : 0.f;
-    at(prm.ngx, z) = -gx;
-    at(prm.ngy, z) = -gy;
-    at(prm.ngzu, z) = -gzu;
-    at(prm.ngzd, z) = -gzd;
-    // diagonal summed in the one-step kernels' order: s, +x, -x, +y, -y, +z, -z
-    for (int nyf = 0; nyf < 3; ++nyf)
-      for (int nxf = 0; nxf < 3; ++nxf) {
-        float dg = sz;
-        dg += nxf >= 1 ? gx : 0.f;
-        dg += nxf >= 2 ? gx : 0.f;
-        dg += nyf >= 1 ? gy : 0.f;
-        dg += nyf >= 2 ? gy : 0.f;
-        dg += gzu;
-        dg += gzd;
-        prm.invd[nxf + 3 * nyf][z] = 1.0f / dg;
-        if (nxf == 2 && nyf == 2) at(prm.d, z) = dg;
-      }
+    const LayerCoefs q = layer_coefs(T, L, z);
+    at(prm.ngx, z) = -q.gx;
+    at(prm.ngy, z) = -q.gy;
+    at(prm.ngzu, z) = -q.gzu;
+    at(prm.ngzd, z) = -q.gzd;
+    at(prm.d, z) = q.d;
+    for (int k = 0; k < 9; ++k) prm.invd[k][z] = q.invd[k];
   }
   CUtensorMap mc, mp, mr;
   TH_TRY(tb_map(&mc, P.d, pool[c.in_cur], EY));
